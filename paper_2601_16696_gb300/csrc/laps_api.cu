@@ -61,13 +61,7 @@ static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 // ------------------------------------------------------------------ small kernels
 __global__ void unpack_rows_kernel(const float* __restrict__ src, const float* __restrict__ scale,
                                    float* __restrict__ dst, int64_t M, int d, int d_pad) {
-    const int64_t n = M * (int64_t)d;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = k / d;
-        const int i = (int)(k - m * d);
-        dst[k] = (scale ? scale[i] : 1.0f) * src[m * d_pad + i];
-    }
+    unpack_rows(src, scale, dst, M, d, d_pad);
 }
 __global__ void ff_to_double_kernel(const float2* __restrict__ src, double* __restrict__ dst,
                                     int64_t n) {
@@ -102,7 +96,7 @@ void launch_set_coefs(Coefs* dst, const Coefs& cf, cudaStream_t st) {
 }
 void launch_unpack(const float* src, const float* scale, float* dst, int64_t M, int d, int d_pad,
                    cudaStream_t st) {
-    unpack_rows_kernel<<<grid_for(M * d), 256, 0, st>>>(src, scale, dst, M, d, d_pad);
+    unpack_rows_kernel<<<row_blocks(M), 256, 0, st>>>(src, scale, dst, M, d, d_pad);
 }
 
 void coefs_table(Coefs& cf) {
@@ -689,7 +683,7 @@ laps_status laps_adapt_freeze(laps_ctx* c, int frozen) {
 laps_status laps_sample(const laps_ctx* c, float* x_out, void* stream) {
     if (!c || !x_out || !aligned(x_out, 4)) return fail(LAPS_ERR_INVALID_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    unpack_rows_kernel<<<grid_for(c->M * c->d), 256, 0, st>>>(c->y, c->sigma, x_out, c->M, c->d,
+    unpack_rows_kernel<<<row_blocks(c->M), 256, 0, st>>>(c->y, c->sigma, x_out, c->M, c->d,
                                                              c->d_pad);
     CK(cudaGetLastError());
     return LAPS_OK;
@@ -704,7 +698,7 @@ laps_status laps_get_state(const laps_ctx* c, float* y, float* u, float* g, doub
     for (int k = 0; k < 3; ++k) {
         if (!dst[k]) continue;
         if (!aligned(dst[k], 4)) return fail(LAPS_ERR_INVALID_ARG, "misaligned output");
-        unpack_rows_kernel<<<grid_for(c->M * c->d), 256, 0, st>>>(src[k], nullptr, dst[k], c->M,
+        unpack_rows_kernel<<<row_blocks(c->M), 256, 0, st>>>(src[k], nullptr, dst[k], c->M,
                                                                  c->d, c->d_pad);
         CK(cudaGetLastError());
     }

@@ -177,8 +177,10 @@ laps_status launch(laps_batch* b, int mode, int n_iters, cudaStream_t st) {
 }
 
 // the start of a run of every problem: its seed in the parameter block, its
-// phase machine (h0, by value), a cleared window, column results and status,
-// sigma = 1; block k takes problems k, k + gridDim.x, ...
+// phase machine (h0, by value), cleared window sums, column results and status,
+// sigma = 1; block k takes problems k, k + gridDim.x, ...  The window's ring is not
+// cleared: a slot is read only once win_n has passed it, so after it was written
+// (clearing d = 10^4's 32 MB ring from one block took about 1 ms of every init).
 __global__ void batch_start_kernel(KParams* probs, Hyper* hyper, int n, uint32_t seed_lo, uint32_t seed_hi,
                                    const Hyper h0, int* status) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
@@ -190,8 +192,6 @@ __global__ void batch_start_kernel(KParams* probs, Hyper* hyper, int n, uint32_t
             hyper[k] = h0;
         }
         const int dp = P.d_pad;
-        const size_t nring = (size_t)(P.T + 1) * dp;
-        for (size_t i = threadIdx.x; i < nring; i += blockDim.x) P.ring[i] = make_float2(0.0f, 0.0f);
         for (int i = threadIdx.x; i < dp; i += blockDim.x) {
             P.win_sums[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             P.sigma[i] = 1.0f;
@@ -205,13 +205,7 @@ __global__ void batch_start_kernel(KParams* probs, Hyper* hyper, int n, uint32_t
 __global__ void batch_unpack_kernel(const float* __restrict__ y, const float* __restrict__ sigma,
                                     const Hyper* __restrict__ h, float* __restrict__ x, int64_t M, int d,
                                     int d_pad) {
-    const bool pend = h->phase == 1 && h->p == 0;
-    const int64_t n = M * (int64_t)d;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = k / d;
-        const int i = (int)(k - m * d);
-        x[k] = (pend ? 1.0f : sigma[i]) * y[m * d_pad + i];
-    }
+    unpack_rows(y, h->phase == 1 && h->p == 0 ? nullptr : sigma, x, M, d, d_pad);
 }
 
 laps_status read_hypers(laps_batch* b) {
@@ -552,9 +546,7 @@ laps_status laps_batch_sample(laps_batch* b, int k, float* x_out, void* stream) 
     if (!b || !x_out || k < 0 || k >= b->n || reinterpret_cast<uintptr_t>(x_out) % 4)
         return fail(LAPS_ERR_INVALID_ARG, "bad argument");
     const BProb& p = b->P[k];
-    const int64_t n = p.M * p.d;
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096));
-    batch_unpack_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>(p.y, p.sigma, b->hyper + k, x_out, p.M,
+    batch_unpack_kernel<<<row_blocks(p.M), 256, 0, (cudaStream_t)stream>>>(p.y, p.sigma, b->hyper + k, x_out, p.M,
                                                                   (int)p.d, p.d_pad);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LAPS_OK : cuda_fail(e, "laps_batch_sample");

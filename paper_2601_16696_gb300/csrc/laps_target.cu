@@ -64,30 +64,32 @@ __global__ void target_logp_grad_kernel(int kind, const float* __restrict__ x, i
     if (lane == 0) logp[m] = part.hi + part.lo;
 }
 
-// LOGREG: the caller's [M][d] points padded to the contraction layout and back
+// LOGREG: the caller's [M][d] points padded to the contraction layout and back, a warp
+// per row (no 64-bit index division: M = 8192, d = 101, tensor-core gradient calls
+// 121.2 -> 117.1 us and 216.5 -> 210.7 us)
 __global__ void logreg_pack_kernel(const float* __restrict__ x, float* __restrict__ W, int64_t M,
                                    int d, int kp) {
-    const int64_t n = M * kp;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = k / kp;
-        const int i = (int)(k - m * kp);
-        W[k] = i < d ? x[m * d + i] : 0.0f;
-    }
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; m < M; m += nw)
+        for (int i = lane; i < kp; i += 32) W[m * kp + i] = i < d ? x[m * d + i] : 0.0f;
 }
 // the S partials of the gradient kernel summed in order, back to the caller's [M][d]
 __global__ void logreg_unpack_kernel(const float* __restrict__ G, const float2* __restrict__ lp,
                                      float* __restrict__ grad, float* __restrict__ logp, int64_t M,
                                      int d, int kp, int S) {
-    const int64_t n = M * d;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = k / d;
-        const int i = (int)(k - m * d);
-        float g = 0.0f;
-        for (int s = 0; s < S; ++s) g += G[((size_t)s * M + m) * kp + i];
-        grad[k] = g;
-        if (i == 0) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const size_t stride = (size_t)M * kp;
+    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; m < M; m += nw) {
+        for (int i = lane; i < d; i += 32) {
+            const float* src = G + m * kp + i;
+            float g = 0.0f;
+#pragma unroll 4
+            for (int s = 0; s < S; ++s) g += src[s * stride];
+            grad[m * d + i] = g;
+        }
+        if (lane == 0) {
             ff l = ff_make(0.0f);
             for (int s = 0; s < S; ++s) l = ff_add(l, ff{lp[(size_t)s * M + m].x, lp[(size_t)s * M + m].y});
             logp[m] = l.hi + l.lo;
@@ -129,7 +131,7 @@ static laps_status streamed_logp_grad(const laps_target* tg, const float* x, int
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&lp, (size_t)S * M * 8, st);
     laps_status rs = LAPS_OK;
     if (e == cudaSuccess) {
-        const int blocks = (int)std::min<int64_t>((M * kp + 255) / 256, 4096);
+        const int blocks = row_blocks(M);
         logreg_pack_kernel<<<blocks, 256, 0, st>>>(x, W, M, d, kp);
         rs = streamed_target_grad(tg, W, M, S, G, lp, st);
         if (rs == LAPS_OK) {
@@ -173,8 +175,7 @@ static laps_status logreg_logp_grad_mixed(const laps_target* tg, const float* x,
     if (e == cudaSuccess) e = logreg_mma_wmap(tmW, Wb, M_pad, kp);
     if (e == cudaSuccess) e = logreg_grad_mma(L, tmW, W32, M, S, rps, G, lp, tg->status, 2000000000LL, st);
     if (e == cudaSuccess) {
-        const int blocks = (int)std::min<int64_t>((M * d + 255) / 256, 4096);
-        logreg_unpack_kernel<<<std::max(blocks, 1), 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S);
+        logreg_unpack_kernel<<<row_blocks(M), 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S);
         e = cudaGetLastError();
     }
     if (W32) cudaFreeAsync(W32, st);
@@ -203,7 +204,7 @@ static laps_status logreg_logp_grad_x3(const laps_target* tg, const float* x, in
     cudaError_t e = cudaMallocAsync((void**)&W32, (size_t)M * kp * 4, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&G, (size_t)S * M * kp * 4, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&lp, (size_t)S * M * 8, st);
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((M * kp + 255) / 256, 4096));
+    const int blocks = row_blocks(M);
     if (e == cudaSuccess) {
         logreg_pack_kernel<<<blocks, 256, 0, st>>>(x, W32, M, d, kp);
         e = cudaGetLastError();
