@@ -174,24 +174,23 @@ logreg_grad_f32_kernel(const float* __restrict__ W, int64_t M, const float* __re
 }
 
 // ---------------------------------------------------------------- packed form
-// The same contraction for kp <= 128 with packed binary32 pairs (fma.rn.f32x2).
-// What bounds it is the FMA pipe: 2 M n d multiply-adds, of which the pipe
-// retires 128 per clock and SM either way, but a packed instruction carries two,
-// so half the issue slots are left for the operand loads and the epilogue.  A
-// thread owns 8 chains x 4 rows of Z and 8 chains x 4 NG columns of G, so that an
-// operand vector from shared memory feeds 8 (4) packed instructions:
-//   Z: pairs along k (even and odd k accumulate apart and are added at the end);
-//      both operands come as pairs from 16-byte loads, and the loop stops at the
-//      last non-zero feature (d rounded up to 4), not at the padded width;
-//   G: pairs along the columns, the residual duplicated into both halves.
-// The epilogue forms log(1 + t) once per four rows, of the product of the four
-// 1 + t (at most 16), and 1 / (1 + t) by the hardware reciprocal with one Newton
-// step.  128 threads and 64 chains per block, two blocks per SM: one block's
-// staging and epilogue overlap the other's contraction.
-// Measured at d = 101, n = 10^4, M = 8192: kernel 1061 -> 804 us, gradient call 1080
-// -> 818 us (FMA pipe 60% -> 69% busy with 23% fewer multiply-adds); error against 64
-// bits unchanged (2.3e-7 of |g|).
-constexpr int PT = 128;  // threads
+// The same contraction for kp <= 128 with packed binary32 pairs (fma.rn.f32x2),
+// every sum in the plain kernel's order (the results are its results).  What bounds
+// it is the FMA pipe: 2 M n d multiply-adds, of which the pipe retires 128 per clock
+// and SM either way, but a packed instruction carries two, so half the issue slots
+// are left for the operand loads and the epilogue.  A thread owns 8 chains x 4 rows
+// of Z and 8 chains x 4 NG columns of G, so that an operand vector from shared
+// memory feeds four to eight packed instructions:
+//   Z: pairs of chains (c, c + 1), interleaved in the W tile; the data value is
+//      duplicated into both halves; the loop stops at the last non-zero feature
+//      (d rounded up to 4), not at the padded width;
+//   G: pairs of columns, the residual stored twice by the epilogue.
+// 128 threads and 64 chains per block, two blocks per SM: one block's staging and
+// epilogue overlap the other's contraction.
+// Measured at d = 101, n = 10^4, M = 8192: gradient call 1083 -> 923 us, same bits
+// (kernel 1061 -> 911 us; FMA pipe 64% busy with 23% fewer multiply-adds in Z).
+constexpr int PT = 128;        // threads
+constexpr int RTP = 2 * TM + 4;  // row stride of the duplicated R tile
 
 template <int KP>
 __global__ void __launch_bounds__(PT, 2)
@@ -199,13 +198,14 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
                         const float* __restrict__ yv, int n, int kz, int rps, float inv_v,
                         float* __restrict__ gpart, float2* __restrict__ lpart, const int* __restrict__ guard) {
     if (guard != nullptr && *guard == 0) return;  // the iteration no longer runs
-    constexpr int LD = KP + 4;   // padded row stride (floats) of the W and X tiles
-    constexpr int NG = KP / 64;  // float4 column groups per thread in the G phase
+    constexpr int LD = KP + 4;       // padded row stride (floats) of the X tile
+    constexpr int LDW = 2 * KP + 4;  // and of the W tile's pairs of rows
+    constexpr int NG = KP / 64;      // float4 column groups per thread in the G phase
     extern __shared__ __align__(16) float sm[];
-    float* Ws = sm;                 // [TM][LD]
-    float* Xs = Ws + TM * LD;       // [TN][LD]
-    float* Rt = Xs + TN * LD;       // [TN][RTS]  Rt[row][8 cr + c]: chain cr + 8 c
-    float* wsq = Rt + TN * RTS;     // [TM] |w|^2
+    float* Ws = sm;                   // [TM / 2][LDW]  row cr + 8 i: chains (cr + 16 i, cr + 16 i + 8), pairs per k
+    float* Xs = Ws + TM / 2 * LDW;    // [TN][LD]
+    float* Rt = Xs + TN * LD;         // [TN][RTP]  Rt[row][32 i + 4 cr]: chain cr + 16 i twice, cr + 16 i + 8 twice
+    float* wsq = Rt + TN * RTP;       // [TM] |w|^2
     ff* s_lp = reinterpret_cast<ff*>(wsq + TM);  // [TM] log p of the upper half of the rows
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -213,22 +213,29 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     const int s = blockIdx.y;
     const int r_begin = s * rps;
     const int r_end = min(n, r_begin + rps);
+    // chain r of the tile at k: row (r & 7) + 8 (r >> 4), half (r >> 3) & 1
+    auto wat = [&](int r, int k) -> float& { return Ws[((r & 7) + 8 * (r >> 4)) * LDW + 2 * k + ((r >> 3) & 1)]; };
 
     // W tile (rows beyond M are zero)
     for (int k = tid; k < TM * (KP / 4); k += PT) {
         const int r = k / (KP / 4), c4 = k - r * (KP / 4);
         float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (m0 + r < M) v = *reinterpret_cast<const float4*>(W + (m0 + r) * KP + 4 * c4);
-        *reinterpret_cast<float4*>(Ws + r * LD + 4 * c4) = v;
+        wat(r, 4 * c4) = v.x;
+        wat(r, 4 * c4 + 1) = v.y;
+        wat(r, 4 * c4 + 2) = v.z;
+        wat(r, 4 * c4 + 3) = v.w;
     }
     __syncthreads();
-    if (s == 0) {  // |w|^2 for the prior term: 2 lanes per chain
-        const int r = tid >> 1, q = tid & 1;
-        float a = 0.0f;
-        for (int k = q; k < KP; k += 2) a = fmaf(Ws[r * LD + k], Ws[r * LD + k], a);
-        a += __shfl_xor_sync(0xffffffffu, a, 1);
-        if (q == 0) wsq[r] = a;
-    }
+    if (s == 0)  // |w|^2 for the prior term: 4 lanes per chain
+        for (int r = tid >> 2; r < TM; r += PT / 4) {
+            const int q = tid & 3;
+            float a = 0.0f;
+            for (int k = q; k < KP; k += 4) a = fmaf(wat(r, k), wat(r, k), a);
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
+            if (q == 0) wsq[r] = a;
+        }
 
     // a warp spans 4 chain groups x 8 rows (columns): its 16-byte operand loads touch
     // 4 or 8 distinct addresses in distinct banks
@@ -242,7 +249,7 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     ff lacc[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) lacc[c] = ff_make(0.0f);
-    const float* wb = Ws + cr * LD;
+    const float* wb = Ws + cr * LDW;
     const float* xb = Xs + dc * LD;
 
     for (int row0 = r_begin; row0 < r_end; row0 += TN) {
@@ -264,67 +271,80 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        // ---- Z = W X^T on the 8 x 4 thread tile
-        f32x2 z[8][4];
+        // ---- Z = W X^T on the 8 x 4 thread tile, k in order
+        f32x2 z[4][4];
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) z[c][e] = 0;
+            for (int e = 0; e < 4; ++e) z[i][e] = 0;
 #pragma unroll 2
         for (int k = 0; k < kz; k += 4) {
-            ulonglong2 xv[4];
+            float4 xv[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xv[e] = *reinterpret_cast<const ulonglong2*>(xb + 16 * e * LD + k);
+            for (int e = 0; e < 4; ++e) xv[e] = *reinterpret_cast<const float4*>(xb + 16 * e * LD + k);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(wb + 8 * c * LD + k);
+            for (int h = 0; h < 2; ++h) {
+                ulonglong2 wv[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) wv[i] = *reinterpret_cast<const ulonglong2*>(wb + 8 * i * LDW + 2 * k + 4 * h);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    z[c][e] = fma2(wv.x, xv[e].x, z[c][e]);
-                    z[c][e] = fma2(wv.y, xv[e].y, z[c][e]);
+                    const float a = h == 0 ? xv[e].x : xv[e].z, b = h == 0 ? xv[e].y : xv[e].w;
+                    const f32x2 aa = pack2(a, a), bb = pack2(b, b);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) z[i][e] = fma2(wv[i].y, bb, fma2(wv[i].x, aa, z[i][e]));
                 }
             }
         }
         // ---- epilogue: residuals and log-likelihood terms
         auto epilogue = [&](auto full) {
-            float lsum[8], lprod[8];
+            float lsum[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) lsum[c] = 0.0f;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool ok = decltype(full)::value || row0 + dc + 16 * e < r_end;
-                float r[8];
+                float4* dst = reinterpret_cast<float4*>(Rt + (dc + 16 * e) * RTP + 4 * cr);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float2 zp = unpack2(z[c][e]);
-                    const float zz = zp.x + zp.y;
-                    const float t = expf(-fabsf(zz));      // e^{-|z|} in (0, 1]
-                    const float opt = 1.0f + t;
-                    float inv;
-                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(opt));
-                    inv = fmaf(inv, fmaf(-opt, inv, 1.0f), inv);
-                    const float sig = zz >= 0.0f ? inv : t * inv;  // sigmoid(z)
-                    // y z - softplus(z) = y z - max(z, 0) - log(1 + t)
-                    const float term = fmaf(yn[e], zz, -fmaxf(zz, 0.0f));
-                    r[c] = ok ? yn[e] - sig : 0.0f;
-                    lsum[c] = (e == 0 ? 0.0f : lsum[c]) + (ok ? term : 0.0f);
-                    lprod[c] = (e == 0 ? 1.0f : lprod[c]) * (ok ? opt : 1.0f);
+                for (int i = 0; i < 4; ++i) {
+                    const float2 zp = unpack2(z[i][e]);
+                    float r[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float zz = h == 0 ? zp.x : zp.y;
+                        const float t = expf(-fabsf(zz));               // e^{-|z|} in (0, 1]
+                        const float sp = fmaxf(zz, 0.0f) + log1pf(t);   // softplus(z)
+                        // 1 / (1 + t): the hardware reciprocal and two Newton steps round as the
+                        // division does for every 1 + t in [1, 2] but 2 - 2^-23 (checked
+                        // exhaustively from starts within two ulps)
+                        const float opt = 1.0f + t;
+                        float inv;
+                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(opt));
+                        inv = fmaf(inv, fmaf(-opt, inv, 1.0f), inv);
+                        inv = fmaf(inv, fmaf(-opt, inv, 1.0f), inv);
+                        const float sig = zz >= 0.0f ? inv : t * inv;   // sigmoid(z)
+                        r[h] = ok ? yn[e] - sig : 0.0f;
+                        lsum[2 * i + h] += ok ? fmaf(yn[e], zz, -sp) : 0.0f;
+                    }
+                    dst[8 * i] = make_float4(r[0], r[0], r[1], r[1]);
                 }
-                float4* dst = reinterpret_cast<float4*>(Rt + (dc + 16 * e) * RTS + 8 * cr);
-                dst[0] = make_float4(r[0], r[1], r[2], r[3]);
-                dst[1] = make_float4(r[4], r[5], r[6], r[7]);
             }
 #pragma unroll
-            for (int c = 0; c < 8; ++c) lacc[c] = ff_add(lacc[c], lsum[c] - logf(lprod[c]));
+            for (int c = 0; c < 8; ++c) lacc[c] = ff_add(lacc[c], lsum[c]);
         };
         if (row0 + TN <= r_end) epilogue(std::true_type{});
         else epilogue(std::false_type{});
         __syncthreads();
-        // ---- G += R^T X over the chunk's rows
+        // ---- G += R^T X over the chunk's rows, in order
 #pragma unroll 2
         for (int r = 0; r < TN; ++r) {
-            const float4 ra = *reinterpret_cast<const float4*>(Rt + r * RTS + 8 * cr);
-            const float4 rb = *reinterpret_cast<const float4*>(Rt + r * RTS + 8 * cr + 4);
-            const f32x2 rr[8] = {pack2(ra.x, ra.x), pack2(ra.y, ra.y), pack2(ra.z, ra.z), pack2(ra.w, ra.w),
-                                 pack2(rb.x, rb.x), pack2(rb.y, rb.y), pack2(rb.z, rb.z), pack2(rb.w, rb.w)};
+            f32x2 rr[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(Rt + r * RTP + 32 * i + 4 * cr);
+                rr[2 * i] = v.x;
+                rr[2 * i + 1] = v.y;
+            }
 #pragma unroll
             for (int q = 0; q < NG; ++q) {
                 const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(Xs + r * LD + 64 * q + 4 * dc);
@@ -355,7 +375,7 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
             const float2 v0 = unpack2(gacc[c][2 * q]), v1 = unpack2(gacc[c][2 * q + 1]);
             float4 v = make_float4(v0.x, v0.y, v1.x, v1.y);
             if (s == 0) {
-                const float4 w = *reinterpret_cast<const float4*>(Ws + (cr + 8 * c) * LD + col);
+                const float4 w = *reinterpret_cast<const float4*>(W + m * KP + col);
                 v.x = fmaf(-w.x, inv_v, v.x);
                 v.y = fmaf(-w.y, inv_v, v.y);
                 v.z = fmaf(-w.z, inv_v, v.z);
@@ -378,8 +398,9 @@ constexpr bool kPacked = KP <= 128;
 
 template <int KP>
 size_t f32_smem() {
-    return ((size_t)TM * (KP + 4) + (size_t)TN * (KP + 4) + (size_t)TN * RTS + TM + (kPacked<KP> ? 2 * TM : 0)) *
-           sizeof(float);
+    const size_t tiles = (size_t)TM * (KP + 4) + (size_t)TN * (KP + 4) + TM;
+    if (kPacked<KP>) return (tiles + (size_t)TN * RTP + 2 * TM) * sizeof(float);  // W: TM / 2 rows of 2 kp + 4
+    return (tiles + (size_t)TN * RTS) * sizeof(float);
 }
 
 template <int KP>
