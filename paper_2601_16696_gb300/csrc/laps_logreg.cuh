@@ -21,12 +21,14 @@ struct LogregData {
     float* y;         // [n] labels
     float inv_v;      // 1 / prior variance
     // tensor-core form (kp <= 128): BF16 copies and their TMA descriptors
-    int n_pad;        // n rounded up to the 64-row chunk
-    void* Xb;         // [n_pad][kp] BF16
-    void* Xtb;        // [kp][n_pad] BF16 (X transposed)
+    void* Xb;         // [n][kp] BF16
+    void* Xf;         // the same with the rows of label 1 negated
+    float* yp;        // [n rounded up to 32] labels in pairs of rows (j, j + 16) of each 32
+    bool bin;         // every label is 0 or 1
     alignas(64) unsigned char tmX[128];   // CUtensorMap of Xb
-    alignas(64) unsigned char tmXt[128];  // CUtensorMap of Xtb
+    alignas(64) unsigned char tmXf[128];  // CUtensorMap of Xf
     // FP32-accurate tensor-core form: the three BF16 terms of X, [3][n_pad][kp]
+    int n_pad;        // n rounded up to the 64-row chunk
     void* X3b;
     alignas(64) unsigned char tmX3[128];  // CUtensorMap of X3b
 };
@@ -36,19 +38,20 @@ constexpr int kLogregMaxKp = 256;
 
 // ---- tensor-core (tcgen05, BF16) gradient: laps_logreg_mma.cu
 bool logreg_mma_supported(int kp);
-// BF16 copies of X and their tensor maps (allocates Xb, Xtb; synchronises)
+// BF16 copies of X, their tensor maps and the paired labels (allocates Xb, Xf, yp; synchronises)
 cudaError_t logreg_mma_prepare(LogregData& D);
 // tensor map of the [M_pad][2 kp] BF16 (hi | lo) copy of the points
 cudaError_t logreg_mma_wmap(void* tmW, const void* Wb, int64_t M_pad, int kp);
-// data splits of the launch (every split non-empty) and rows per split
-int logreg_mma_splits(const LogregData& D, int64_t M, int nsm, int* rps);
+// data splits of the launch (every split non-empty) and rows per split.  fold: the
+// form of target calls on labels in {0, 1} (D.bin); else the sampler's
+int logreg_mma_splits(const LogregData& D, int64_t M, int nsm, bool fold, int* rps);
 // points [M][d] -> FP32 [M][kp] and BF16 hi | lo [M_pad][2 kp] (rows past M untouched)
 cudaError_t logreg_pack_points(const float* x, int64_t M, int d, int kp, float* W32, void* Wb,
                                cudaStream_t st);
 // gradient partials like logreg_grad_f32; W32 is the FP32 [M][kp] copy of the
 // points (prior terms); a bounded wait that expires sets *status
 cudaError_t logreg_grad_mma(const LogregData& D, const void* tmW, const float* W32, int64_t M, int S,
-                            int rps, float* gpart, float2* lpart, int* status, long long timeout_ns,
+                            int rps, bool fold, float* gpart, float2* lpart, int* status, long long timeout_ns,
                             cudaStream_t st, const int* guard = nullptr);
 
 // ---- tensor-core gradient at FP32 accuracy (three-term BF16 split): laps_logreg_x3.cu

@@ -3,25 +3,41 @@
 // tensor memory), for the unadjusted phase of the mixed-precision form.
 //
 // A CTA owns 128 chains (one MMA M tile) and one range of data rows, which it
-// walks in chunks of 64 rows:
-//   Z_c  = [W_hi | W_lo] [X_c | X_c]^T     128 x 64, K = 2 kp   (TMEM, two buffers)
+// walks in chunks of 128 rows:
+//   Z_c  = [W_hi | W_lo] [X_c | X_c]^T     128 x 128, K = 2 d   (TMEM, two buffers)
 //   R_c  = y_c - sigmoid(Z_c)  (BF16, written into tensor memory by the epilogue)
-//   G   += R_c X_c                          128 x kp, K = 64     (TMEM; R read from TMEM)
+//   G   += R_c X_c                          128 x d, K = 128     (TMEM; R read from TMEM)
 // W = x is split into two BF16 terms (hi + lo carries ~16 significant bits),
 // so the logits are those of the BF16-rounded data at nearly FP32 accuracy in
 // x and log p stays smooth along a trajectory; R is a single BF16 term.
 //
-// Roles (640 threads): warp 0 loads W once and X / X^T chunks through a
-// 4-stage ring with TMA (128-byte swizzle); warp 1 issues the MMAs from one
-// thread; warps 4..19 are the epilogue (warp w reads TMEM lanes 32 (w % 4) ..
-// +31, i.e. chains, and a quarter of the columns).  All waits are bounded: on
-// expiry the CTA records ST_TIMEOUT in the status word, drains what it
-// issued and frees its tensor memory.
+// Two epilogues.  The sampler's (FOLD = false) takes every row's logarithm and adds
+// sixteen rows' terms in order, so that a run's log p does not depend on how rows are
+// paired here; pairs of rows (j, j + 16) go through packed arithmetic side by side.  A
+// target call on labels in {0, 1} (FOLD = true) rounds log p to binary32 anyway: it reads
+// a copy of X whose label-1 rows are negated (exact), so that with z'' = (1 - 2 y) z the
+// term is -softplus(z'') and the residual sigmoid(z''), loads no labels and takes one
+// logarithm per sixteen rows, of the product of their 1 + t.
+//
+// What bounds it: the epilogue's special-function unit (ex2, reciprocal and, for the
+// sampler, a logarithm per logit: 1/32 + 1/16 + 1/16 clocks and SM) and issue slots,
+// next to the tensor pipe.  K and N stop at d rounded up to 16, not at the padded width;
+// Z products of N = 128 run at the tensor peak, N = 64 ones at 63% of it; one copy of a
+// data chunk serves both products (K-major for Z, MN-major for G).
+// Measured at d = 101, n = 10^4, M = 8192 (kernel time; 64-row chunks, two copies of a
+// chunk and scalar epilogue before): target call 105 -> 76 us, sampler 105 -> 86 us.
+//
+// Roles (640 threads): warp 0 loads W once and X chunks through a 4-stage ring
+// with TMA (128-byte swizzle); warp 1 issues the MMAs from one thread; warps
+// 4..19 are the epilogue (warp w reads TMEM lanes 32 (w % 4) .. +31, i.e. chains,
+// and a quarter of the columns).  All waits are bounded: on expiry the CTA records
+// ST_TIMEOUT in the status word, drains what it issued and frees its tensor memory.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "laps_device.cuh"
 #include "laps_logreg.cuh"
@@ -32,8 +48,8 @@ namespace laps {
 namespace {
 
 constexpr int MT = 128;      // chains per CTA (MMA M)
-constexpr int TNR = 64;      // data rows per chunk (MMA N of Z, K of G)
-constexpr int NSTAGE = 4;    // X / X^T ring depth
+constexpr int TNR = 128;     // data rows per chunk (MMA N of Z, K of G)
+constexpr int NSTAGE = 4;    // X ring depth
 constexpr int NTHR = 640;
 constexpr int EPI_WARP0 = 4;  // first epilogue warp
 constexpr int NEPI = 16;      // epilogue warps: 4 lane quarters x 4 column quarters
@@ -66,10 +82,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 struct MmaArgs {
     int64_t M;           // chains
     int n;               // data rows
-    int rps;             // rows per split, a multiple of 64
+    int rps;             // rows per split, a multiple of 64 (FOLD: of TNR)
+    int d;               // features (padding columns of X and W are zero)
     float inv_v;         // 1 / prior variance
     const float* W32;    // [M][kp] FP32 x (for the prior terms)
-    const float* y;      // [n] labels
+    const float* yp;     // labels in pairs: 32 g + 2 j + {0, 1} holds rows 32 g + j and 32 g + 16 + j
     float* gpart;        // [S][M][kp]
     float2* lpart;       // [S][M]
     int* status;
@@ -81,28 +98,28 @@ template <int KP>
 struct Smem {
     static constexpr int NA = KP / 64;                    // 64-wide K atoms of one W term
     static constexpr uint32_t W_BYTES = 2u * NA * MT * 128;  // hi and lo
-    static constexpr uint32_t X_BYTES = (uint32_t)NA * TNR * 128;
-    static constexpr uint32_t XT_BYTES = (uint32_t)KP * 128;
-    static constexpr uint32_t STAGE = X_BYTES + XT_BYTES;
+    static constexpr uint32_t ATOM = (uint32_t)TNR * 128;     // 64 features of one chunk
+    static constexpr uint32_t STAGE = (uint32_t)NA * ATOM;
     static constexpr uint32_t OFF_W = 0;
     static constexpr uint32_t OFF_X = OFF_W + W_BYTES;
     static constexpr uint32_t OFF_BAR = OFF_X + NSTAGE * STAGE;
     static constexpr uint32_t OFF_LP = OFF_BAR + 256;      // [4][MT] float-float
     static constexpr uint32_t TOTAL = OFF_LP + 4 * MT * 8 + 1024;  // + alignment slack
-    // tensor memory: Z buffers [0, 128), G [128, 128 + kp), R buffers (64 BF16 rows
-    // per chain = 32 columns each) after G
-    static constexpr uint32_t T_R = 2 * TNR + KP, TMEM_COLS = T_R + 2 * (TNR / 2) <= 256 ? 256 : 512;
+    // tensor memory: Z buffers [0, 256), G [256, 256 + kp), R buffers (128 BF16 rows
+    // per chain = 64 columns each) after G
+    static constexpr uint32_t T_R = 2 * TNR + KP, TMEM_COLS = 512;
     static_assert(T_R + TNR <= TMEM_COLS, "tensor memory columns");
+    static_assert(TOTAL <= 227 * 1024, "shared memory");
 };
 
 enum { B_WFULL = 0, B_XFULL = 1, B_XEMPTY = B_XFULL + NSTAGE, B_ZFULL = B_XEMPTY + NSTAGE,
        B_ZEMPTY = B_ZFULL + 2, B_RFULL = B_ZEMPTY + 2, B_REMPTY = B_RFULL + 2,
        B_GDONE = B_REMPTY + 2, B_DRAIN = B_GDONE + 1, NBAR = B_DRAIN + 1 };
 
-template <int KP>
+template <int KP, bool FOLD>
 __global__ void __launch_bounds__(NTHR, 1)
 logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-                       const __grid_constant__ CUtensorMap tmXt, const MmaArgs A) {
+                       const MmaArgs A) {
     if (A.guard != nullptr && *A.guard == 0) return;  // uniform: before any barrier or allocation
     using S = Smem<KP>;
     extern __shared__ __align__(1024) unsigned char mma_smem_raw[];
@@ -168,8 +185,7 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
             mbar_expect_tx(bar(B_XFULL + st), S::STAGE);
             const int row = r_begin + c * TNR;
             for (int a = 0; a < S::NA; ++a)
-                tma_load_2d(dst + (uint32_t)a * (TNR * 128), &tmX, 64 * a, row, bar(B_XFULL + st));
-            tma_load_2d(dst + S::X_BYTES, &tmXt, row, 0, bar(B_XFULL + st));
+                tma_load_2d(dst + (uint32_t)a * S::ATOM, &tmX, 64 * a, row, bar(B_XFULL + st));  // rows past n: 0
             issued = c + 1;
         }
         if (!ok) {
@@ -185,7 +201,10 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
     } else if (warp == 1) {
       if (lane == 0) {
         // ------------------------------------------------ MMA issuer
-        constexpr uint32_t ID_Z = idesc_bf16(MT, TNR), ID_G = idesc_bf16(MT, KP);
+        constexpr uint32_t ID_Z = idesc_bf16(MT, TNR);
+        const int k16 = (A.d + 15) / 16;  // K steps of one term of Z; N of G
+        const uint32_t ID_G = idesc_bf16(MT, 16 * k16, true);
+        const uint64_t dX = sw128_desc(sX), dXmn = sw128_mn_desc(sX, S::ATOM), dW = sw128_desc(sW);
         bool ok = mbar_wait(bar(B_WFULL), 0, deadline);
         tc_fence_after();
         auto gemm2 = [&](int cc) -> bool {
@@ -193,11 +212,10 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
             if (!mbar_wait(bar(B_RFULL + rb), (cc >> 1) & 1, deadline)) return false;
             tc_fence_after();
             const uint32_t aR = tR + (uint32_t)rb * (TNR / 2);
-            const uint32_t bXt = sX + (uint32_t)st * S::STAGE + S::X_BYTES;
+            const uint64_t bX = dXmn + (uint64_t)((uint32_t)st * S::STAGE >> 4);
 #pragma unroll
             for (int kk = 0; kk < TNR / 16; ++kk)
-                tc_mma_ts(tG, aR + 8u * kk, sw128_desc(bXt + 32u * kk), ID_G,
-                       (cc > 0 || kk > 0) ? 1u : 0u);
+                tc_mma_ts(tG, aR + 8u * kk, bX + (2048u * kk >> 4), ID_G, (cc > 0 || kk > 0) ? 1u : 0u);
             tc_commit(bar(B_REMPTY + rb));
             tc_commit(bar(B_XEMPTY + st));
             return true;
@@ -211,17 +229,16 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
                     break;
                 }
                 tc_fence_after();
-                const uint32_t bX = sX + (uint32_t)st * S::STAGE;
+                const uint64_t bX = dX + (uint64_t)((uint32_t)st * S::STAGE >> 4);
                 const uint32_t dZ = tZ + (uint32_t)zb * TNR;
-                int k = 0;
 #pragma unroll
                 for (int part = 0; part < 2; ++part)
 #pragma unroll
-                    for (int kk = 0; kk < KP / 16; ++kk, ++k) {
-                        const uint32_t aW = sW + (uint32_t)(part * S::NA + kk / 4) * (MT * 128) + 32u * (kk % 4);
-                        const uint32_t bx = bX + (uint32_t)(kk / 4) * (TNR * 128) + 32u * (kk % 4);
-                        tc_mma(dZ, sw128_desc(aW), sw128_desc(bx), ID_Z, k > 0 ? 1u : 0u);
-                    }
+                    for (int kk = 0; kk < KP / 16; ++kk)
+                        if (kk < k16)
+                            tc_mma(dZ, dW + (((uint32_t)(part * S::NA + kk / 4) * (MT * 128) + 32u * (kk % 4)) >> 4),
+                                   bX + (((uint32_t)(kk / 4) * S::ATOM + 32u * (kk % 4)) >> 4), ID_Z,
+                                   part + kk > 0 ? 1u : 0u);
                 tc_commit(bar(B_ZFULL + zb));
             }
             if (c >= 1 && !gemm2(c - 1)) { ok = false; break; }
@@ -238,68 +255,95 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
     } else if (warp >= EPI_WARP0 && warp < EPI_WARP0 + NEPI) {
         // ------------------------------------------------ epilogue
         const int q = warp & 3;                 // TMEM lane quarter: chains 32q .. 32q+31
-        const int h = (warp - EPI_WARP0) >> 2;  // column quarter: Z columns 16h .. 16h+15
+        constexpr int ZC = TNR / 4;             // Z columns of one warp
+        const int h = (warp - EPI_WARP0) >> 2;  // column quarter: Z columns ZC h .. ZC h + ZC - 1
         const int rt = 32 * q + lane;           // this thread's chain in the tile
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
+        const f32x2 one2 = pack2(1.0f, 1.0f), m1 = pack2(-1.0f, -1.0f);
+        const f32x2 nln2 = pack2(-0.6931471805599453f, -0.6931471805599453f);
         ff lp = ff_make(0.0f);
         bool ok = true;
         for (int c = 0; c < nc; ++c) {
             const int zb = c & 1;
-            // the labels of data rows row0 .. row0 + 15, loaded before waiting for Z
-            const int row0 = r_begin + c * TNR + 16 * h;
-            const int nlive = min(16, r_end - row0);
-            float yy[16];
-            if (nlive >= 16) {
-#pragma unroll
-                for (int j4 = 0; j4 < 4; ++j4) {
-                    const float4 v = __ldg(reinterpret_cast<const float4*>(A.y + row0) + j4);
-                    yy[4 * j4] = v.x; yy[4 * j4 + 1] = v.y; yy[4 * j4 + 2] = v.z; yy[4 * j4 + 3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) yy[j] = j < nlive ? A.y[row0 + j] : 0.0f;
-            }
+            const int row0 = r_begin + c * TNR + ZC * h;
+            const int nlive = min(ZC, max(0, r_end - row0));
             if (!mbar_wait(bar(B_ZFULL + zb), (c >> 1) & 1, deadline)) { ok = false; break; }
             tc_fence_after();
-            float z[16];
-            tmem_ld16(tZ + lane_off + (uint32_t)(zb * TNR + 16 * h), z);
+            float z[ZC];
+            tmem_ld32(tZ + lane_off + (uint32_t)(zb * TNR + ZC * h), z);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_ZEMPTY + zb));
-            // residuals and log-likelihood terms.  Fast SFU approximations (this
-            // form serves the unadjusted phase only): t = e^{-|z|}, sigmoid from
-            // 1 / (1 + t), softplus = max(z, 0) + log(1 + t)
-            float r[16];
-            float lsum = 0.0f;
-            auto body = [&](auto full) {
+            // Fast SFU approximations (this form serves the unadjusted phase only):
+            // t = e^{-|z|}, sigmoid = (z >= 0 ? 1 : t) / (1 + t), softplus = max(z, 0) +
+            // log(1 + t)
+            uint32_t pr[ZC / 2];
+            if constexpr (FOLD) {
+                // Rows past n have z = 0 exactly: their sigmoid meets a zero data row, their
+                // log 2 is taken off below.  The pairs' halves accumulate apart.
+                f32x2 prod = one2, msum = 0;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const float zz = z[j];
-                    const float t = ex2_ftz(-1.4426950408889634f * fabsf(zz));  // e^{-|z|}
-                    const float opt = 1.0f + t;
-                    const float inv = rcp_ftz(opt);
-                    const float sig = zz >= 0.0f ? inv : t * inv;
-                    const float sp = fmaf(0.6931471805599453f, lg2_ftz(opt), fmaxf(zz, 0.0f));
-                    const float term = fmaf(yy[j], zz, -sp);
-                    if (decltype(full)::value) {
-                        r[j] = yy[j] - sig;
-                        lsum += term;
-                    } else {
-                        r[j] = j < nlive ? yy[j] - sig : 0.0f;
-                        lsum += j < nlive ? term : 0.0f;
-                    }
+                for (int j = 0; j < ZC; j += 2) {
+                    const float t0 = ex2_ftz(-1.4426950408889634f * fabsf(z[j]));
+                    const float t1 = ex2_ftz(-1.4426950408889634f * fabsf(z[j + 1]));
+                    const f32x2 opt = add2(pack2(t0, t1), one2);
+                    const float2 o = unpack2(opt);
+                    const float2 r = unpack2(mul2(pack2(z[j] >= 0.0f ? 1.0f : t0, z[j + 1] >= 0.0f ? 1.0f : t1),
+                                                  pack2(rcp_ftz(o.x), rcp_ftz(o.y))));
+                    prod = mul2(prod, opt);
+                    msum = add2(msum, pack2(fmaxf(z[j], 0.0f), fmaxf(z[j + 1], 0.0f)));
+                    pr[j / 2] = pack_bf16(-r.x, -r.y);
                 }
-            };
-            if (nlive >= 16) body(std::true_type{});
-            else body(std::false_type{});
-            lp = ff_add(lp, lsum);
+                const float2 ps = unpack2(prod), ms = unpack2(msum);
+                const float l0 = fmaf(0.6931471805599453f, lg2_ftz(ps.x) - (float)((ZC - nlive) / 2), ms.x);
+                const float l1 = fmaf(0.6931471805599453f, lg2_ftz(ps.y) - (float)((ZC - nlive + 1) / 2), ms.y);
+                lp = ff_add(ff_add(lp, -l0), -l1);
+            } else {
+                f32x2 lsum = 0;  // rows row0 .. + 15 and row0 + 16 .. + 31, each in order
+                const ulonglong2* yp = reinterpret_cast<const ulonglong2*>(A.yp + row0);
+                auto body = [&](auto full) {
+#pragma unroll
+                    for (int j = 0; j < ZC / 2; j += 2) {
+                        f32x2 yy[2] = {0, 0}, rr[2];
+                        if (decltype(full)::value || nlive > j) {
+                            const ulonglong2 v = __ldg(yp + j / 2);
+                            yy[0] = v.x;
+                            yy[1] = v.y;
+                        }
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float z0 = z[j + e], z1 = z[j + e + ZC / 2];
+                            const float t0 = ex2_ftz(-1.4426950408889634f * fabsf(z0));
+                            const float t1 = ex2_ftz(-1.4426950408889634f * fabsf(z1));
+                            const float2 o = unpack2(add2(pack2(t0, t1), one2));
+                            const f32x2 sig = mul2(pack2(z0 >= 0.0f ? 1.0f : t0, z1 >= 0.0f ? 1.0f : t1),
+                                                   pack2(rcp_ftz(o.x), rcp_ftz(o.y)));
+                            const f32x2 nsp = fma2(pack2(lg2_ftz(o.x), lg2_ftz(o.y)), nln2,
+                                                   pack2(fminf(-z0, 0.0f), fminf(-z1, 0.0f)));  // -softplus
+                            f32x2 term = fma2(yy[e], pack2(z0, z1), nsp);
+                            rr[e] = fma2(sig, m1, yy[e]);  // y - sigmoid
+                            if (!decltype(full)::value) {  // rows past the range add nothing
+                                const float2 tv = unpack2(term), rv = unpack2(rr[e]);
+                                const bool a = j + e < nlive, b = j + e + ZC / 2 < nlive;
+                                term = pack2(a ? tv.x : 0.0f, b ? tv.y : 0.0f);
+                                rr[e] = pack2(a ? rv.x : 0.0f, b ? rv.y : 0.0f);
+                            }
+                            lsum = add2(lsum, term);
+                        }
+                        const float2 r0 = unpack2(rr[0]), r1 = unpack2(rr[1]);
+                        pr[j / 2] = pack_bf16(r0.x, r1.x);
+                        pr[j / 2 + ZC / 4] = pack_bf16(r0.y, r1.y);
+                    }
+                };
+                if (nlive == ZC) body(std::true_type{});
+                else body(std::false_type{});
+                const float2 ls = unpack2(lsum);
+                lp = ff_add(ff_add(lp, ls.x), ls.y);
+            }
             const int rb = zb;
             if (!mbar_wait(bar(B_REMPTY + rb), ((c >> 1) & 1) ^ 1, deadline)) { ok = false; break; }
-            // R row rt, data rows 16h .. 16h+15: columns 8h .. 8h+7 of this lane's R buffer
-            uint32_t pr[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) pr[e] = pack_bf16(r[2 * e], r[2 * e + 1]);
-            tmem_st8(tR + lane_off + (uint32_t)(rb * (TNR / 2) + 8 * h), pr);
+            // R row rt, data rows ZC h .. ZC h + ZC - 1: columns ZC/2 h .. of this lane's R buffer
+            tmem_st16(tR + lane_off + (uint32_t)(rb * (TNR / 2) + (ZC / 2) * h), pr);
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
@@ -319,9 +363,9 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
                 float g[16];
                 const int col = h * (KP / 4) + 16 * piece;
                 tmem_ld16(tG + lane_off + (uint32_t)col, g);
-                if (nc == 0)
+                if (nc == 0 || col >= A.d)  // no chunk, or past the products' N (d rounded up to 16)
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) g[k] = 0.0f;  // no chunk: G was never written
+                    for (int k = 0; k < 16; ++k) g[k] = 0.0f;  // G was never written
                 if (m < A.M) {
 #pragma unroll
                     for (int j4 = 0; j4 < 4; ++j4) {
@@ -369,15 +413,24 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
 }
 
 // ------------------------------------------------------------------ host
-__global__ void to_bf16_kernel(const float* __restrict__ X, __nv_bfloat16* __restrict__ Xb,
-                               __nv_bfloat16* __restrict__ Xtb, int n, int n_pad, int kp) {
-    const int64_t tot = (int64_t)n_pad * kp;
+// X in BF16 and, in Xf, the same with the rows of label 1 negated
+__global__ void to_bf16_kernel(const float* __restrict__ X, const float* __restrict__ y, __nv_bfloat16* __restrict__ Xb,
+                               __nv_bfloat16* __restrict__ Xf, int n, int kp) {
+    const int64_t tot = (int64_t)n * kp;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < tot;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(k / kp), i = (int)(k - (int64_t)r * kp);
-        const __nv_bfloat16 v = __float2bfloat16_rn(r < n ? X[(size_t)r * kp + i] : 0.0f);
+        const __nv_bfloat16 v = __float2bfloat16_rn(X[k]);
         Xb[k] = v;
-        Xtb[(size_t)i * n_pad + r] = v;
+        Xf[k] = y[k / kp] == 1.0f ? __hneg(v) : v;
+    }
+}
+// the labels in pairs (rows past n: 0); *other = 1 if some label is neither 0 nor 1
+__global__ void pair_labels_kernel(const float* __restrict__ y, int n, int n32, float* __restrict__ yp,
+                                   int* __restrict__ other) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n32; k += gridDim.x * blockDim.x) {
+        const float v = k < n ? y[k] : 0.0f;
+        yp[(k & ~31) + 2 * (k & 15) + ((k >> 4) & 1)] = v;
+        if (!(v == 0.0f || v == 1.0f)) *other = 1;
     }
 }
 
@@ -394,6 +447,15 @@ __global__ void pack_points_kernel(const float* __restrict__ x, int64_t M, int d
             Wb[m * 2 * kp + i] = hi;
             Wb[m * 2 * kp + kp + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
         }
+}
+
+template <int KP, bool FOLD>
+cudaError_t launch_mma(const CUtensorMap& mw, const CUtensorMap& mx, const MmaArgs& a, dim3 grid, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(logreg_grad_mma_kernel<KP, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Smem<KP>::TOTAL);
+    if (e != cudaSuccess) return e;
+    logreg_grad_mma_kernel<KP, FOLD><<<grid, NTHR, Smem<KP>::TOTAL, st>>>(mw, mx, a);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -414,34 +476,30 @@ cudaError_t logreg_mma_prepare(LogregData& D) {
     if (!logreg_mma_supported(D.kp)) return cudaErrorInvalidValue;
     EncodeTiled enc = encoder();
     if (!enc) return cudaErrorNotSupported;
-    D.n_pad = (D.n + TNR - 1) / TNR * TNR;
-    const size_t nb = (size_t)D.n_pad * D.kp * sizeof(__nv_bfloat16);
+    const size_t nb = (size_t)D.n * D.kp * sizeof(__nv_bfloat16);
+    const int n32 = (D.n + 31) / 32 * 32;
+    int* other = nullptr;
     cudaError_t e = cudaMalloc(&D.Xb, nb);
-    if (e == cudaSuccess) e = cudaMalloc(&D.Xtb, nb);
+    if (e == cudaSuccess) e = cudaMalloc(&D.Xf, nb);
+    if (e == cudaSuccess) e = cudaMalloc(&D.yp, (size_t)n32 * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&other, sizeof(int));
     if (e != cudaSuccess) return e;
-    to_bf16_kernel<<<std::min(4096, (int)((D.n_pad * (int64_t)D.kp + 255) / 256)), 256>>>(
-        D.X, reinterpret_cast<__nv_bfloat16*>(D.Xb), reinterpret_cast<__nv_bfloat16*>(D.Xtb), D.n, D.n_pad, D.kp);
-    e = cudaGetLastError();
+    int h_other = 0;
+    e = cudaMemset(other, 0, sizeof(int));
+    if (e == cudaSuccess) {
+        pair_labels_kernel<<<std::min(1024, (n32 + 255) / 256), 256>>>(D.y, D.n, n32, D.yp, other);
+        to_bf16_kernel<<<std::min(4096, (int)((D.n * (int64_t)D.kp + 255) / 256)), 256>>>(
+            D.X, D.y, reinterpret_cast<__nv_bfloat16*>(D.Xb), reinterpret_cast<__nv_bfloat16*>(D.Xf), D.n, D.kp);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(&h_other, other, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(other);
     if (e != cudaSuccess) return e;
-    const cuuint32_t es[2] = {1, 1};
-    {   // X: [n_pad][kp], boxes of 64 features x 64 rows
-        const cuuint64_t dims[2] = {(cuuint64_t)D.kp, (cuuint64_t)D.n_pad};
-        const cuuint64_t strides[1] = {(cuuint64_t)D.kp * 2};
-        const cuuint32_t box[2] = {64, TNR};
-        if (enc(reinterpret_cast<CUtensorMap*>(D.tmX), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, D.Xb, dims, strides,
-                box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
-    {   // X^T: [kp][n_pad], boxes of 64 rows x kp features
-        const cuuint64_t dims[2] = {(cuuint64_t)D.n_pad, (cuuint64_t)D.kp};
-        const cuuint64_t strides[1] = {(cuuint64_t)D.n_pad * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)D.kp};
-        if (enc(reinterpret_cast<CUtensorMap*>(D.tmXt), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, D.Xtb, dims, strides,
-                box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
+    D.bin = h_other == 0;
+    // [n][kp], boxes of 64 features x 128 rows (rows past n read as zero)
+    if (!encode_bf16_2d(D.tmX, D.Xb, (uint64_t)D.kp, (uint64_t)D.n, 64, TNR) ||
+        !encode_bf16_2d(D.tmXf, D.Xf, (uint64_t)D.kp, (uint64_t)D.n, 64, TNR))
+        return cudaErrorInvalidValue;
     return cudaDeviceSynchronize();
 }
 
@@ -459,28 +517,30 @@ cudaError_t logreg_mma_wmap(void* tmW, const void* Wb, int64_t M_pad, int kp) {
     return cudaSuccess;
 }
 
-int logreg_mma_splits(const LogregData& D, int64_t M, int nsm, int* rps_out) {
+int logreg_mma_splits(const LogregData& D, int64_t M, int nsm, bool fold, int* rps_out) {
     const int64_t tiles = (M + MT - 1) / MT;
+    const int unit = fold ? TNR : 64;
     int S = (int)std::max<int64_t>(1, nsm / std::max<int64_t>(1, tiles));
-    const int chunks = (D.n + TNR - 1) / TNR;
+    const int chunks = (D.n + unit - 1) / unit;
     S = std::max(1, std::min(S, chunks));
-    int rps = ((D.n + S - 1) / S + TNR - 1) / TNR * TNR;
+    int rps = ((D.n + S - 1) / S + unit - 1) / unit * unit;
     S = (D.n + rps - 1) / rps;
     if (rps_out) *rps_out = rps;
     return S;
 }
 
 cudaError_t logreg_grad_mma(const LogregData& D, const void* tmW, const float* W32, int64_t M, int S,
-                            int rps, float* gpart, float2* lpart, int* status, long long timeout_ns,
+                            int rps, bool fold, float* gpart, float2* lpart, int* status, long long timeout_ns,
                             cudaStream_t st, const int* guard) {
     if (M <= 0) return cudaSuccess;
     MmaArgs a;
     a.M = M;
     a.n = D.n;
+    a.d = D.d;
     a.rps = rps;
     a.inv_v = D.inv_v;
     a.W32 = W32;
-    a.y = D.y;
+    a.yp = D.yp;
     a.gpart = gpart;
     a.lpart = lpart;
     a.status = status;
@@ -488,23 +548,11 @@ cudaError_t logreg_grad_mma(const LogregData& D, const void* tmW, const float* W
     a.guard = guard;
     const dim3 grid((unsigned)((M + MT - 1) / MT), (unsigned)S);
     const CUtensorMap& mw = *reinterpret_cast<const CUtensorMap*>(tmW);
-    const CUtensorMap& mx = *reinterpret_cast<const CUtensorMap*>(D.tmX);
-    const CUtensorMap& mt = *reinterpret_cast<const CUtensorMap*>(D.tmXt);
-    cudaError_t e;
-    if (D.kp == 64) {
-        e = cudaFuncSetAttribute(logreg_grad_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)Smem<64>::TOTAL);
-        if (e != cudaSuccess) return e;
-        logreg_grad_mma_kernel<64><<<grid, NTHR, Smem<64>::TOTAL, st>>>(mw, mx, mt, a);
-    } else if (D.kp == 128) {
-        e = cudaFuncSetAttribute(logreg_grad_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)Smem<128>::TOTAL);
-        if (e != cudaSuccess) return e;
-        logreg_grad_mma_kernel<128><<<grid, NTHR, Smem<128>::TOTAL, st>>>(mw, mx, mt, a);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    const CUtensorMap& mx = *reinterpret_cast<const CUtensorMap*>(fold ? D.tmXf : D.tmX);
+    if (D.kp == 64) return fold ? launch_mma<64, true>(mw, mx, a, grid, st) : launch_mma<64, false>(mw, mx, a, grid, st);
+    if (D.kp == 128)
+        return fold ? launch_mma<128, true>(mw, mx, a, grid, st) : launch_mma<128, false>(mw, mx, a, grid, st);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace laps

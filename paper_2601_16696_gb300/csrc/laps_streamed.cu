@@ -434,7 +434,7 @@ laps_status launch_grad(laps_ctx* c, int form, cudaStream_t st, const int* guard
     }
     if (c->tg->kind == TGT_USER) return user_grad(c->tg, c->W, c->M, c->d_pad, c->gpart, c->ulp, c->lpart, st);
     if (form == GF_BF16)
-        e = logreg_grad_mma(c->tg->lr, c->tmW, c->W, c->M, c->nsplit_mma, c->rps_mma, c->gpart, c->lpart,
+        e = logreg_grad_mma(c->tg->lr, c->tmW, c->W, c->M, c->nsplit_mma, c->rps_mma, false, c->gpart, c->lpart,
                             c->status, c->cfg.barrier_timeout_ns, st, guard);
     else if (form == GF_X3)
         e = logreg_grad_x3(c->tg->lr, c->W, c->M, c->nsplit_x3, c->rps_x3, c->gpart, c->lpart, c->status,
@@ -603,7 +603,7 @@ laps_status streamed_setup(laps_ctx* c) {
     if (c->gf_adj == GF_X3 && (!logreg_x3_supported(dp) || c->tg->lr.X3b == nullptr))
         return fail(LAPS_ERR_UNSUPPORTED, "the three-term tensor-core form is built for LOGREG with d <= 128");
     c->mixed = c->gf_unadj == GF_BF16;
-    if (c->gf_unadj == GF_BF16) c->nsplit_mma = logreg_mma_splits(c->tg->lr, c->M, nsm, &c->rps_mma);
+    if (c->gf_unadj == GF_BF16) c->nsplit_mma = logreg_mma_splits(c->tg->lr, c->M, nsm, false, &c->rps_mma);
     if (c->gf_unadj == GF_X3 || c->gf_adj == GF_X3)
         c->nsplit_x3 = logreg_x3_splits(c->tg->lr, c->M, nsm, &c->rps_x3);
     if (c->mixed) c->M_pad = (c->M + 127) / 128 * 128;

@@ -159,7 +159,7 @@ static laps_status logreg_logp_grad_mixed(const laps_target* tg, const float* x,
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     int rps = 64;
-    const int S = logreg_mma_splits(L, M, nsm, &rps);
+    const int S = logreg_mma_splits(L, M, nsm, L.bin, &rps);
     float *W32 = nullptr, *G = nullptr;
     void* Wb = nullptr;
     float2* lp = nullptr;
@@ -173,7 +173,7 @@ static laps_status logreg_logp_grad_mixed(const laps_target* tg, const float* x,
                             (size_t)(M_pad - M) * 2 * kp * 2, st);
     if (e == cudaSuccess) e = logreg_pack_points(x, M, d, kp, W32, Wb, st);
     if (e == cudaSuccess) e = logreg_mma_wmap(tmW, Wb, M_pad, kp);
-    if (e == cudaSuccess) e = logreg_grad_mma(L, tmW, W32, M, S, rps, G, lp, tg->status, 2000000000LL, st);
+    if (e == cudaSuccess) e = logreg_grad_mma(L, tmW, W32, M, S, rps, L.bin, G, lp, tg->status, 2000000000LL, st);
     if (e == cudaSuccess) {
         logreg_unpack_kernel<<<row_blocks(M), 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S);
         e = cudaGetLastError();
