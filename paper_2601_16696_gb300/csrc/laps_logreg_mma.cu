@@ -24,13 +24,15 @@
 // next to the tensor pipe.  K and N stop at d rounded up to 16, not at the padded width;
 // Z products of N = 128 run at the tensor peak, N = 64 ones at 63% of it; one copy of a
 // data chunk serves both products (K-major for Z, MN-major for G).
-// Measured at d = 101, n = 10^4, M = 8192 (kernel time; 64-row chunks, two copies of a
-// chunk and scalar epilogue before): target call 105 -> 76 us, sampler 105 -> 86 us.
+// Measured at d = 101, n = 10^4, M = 8192 (kernel time): 105 us with 64-row chunks, two
+// copies of a chunk, a scalar epilogue and one issuing thread; target call 76 us, sampler
+// 86 us with the above; 60 and 81 us with an issuing warp per chain and two epilogue groups.
 //
 // Roles (640 threads): warp 0 loads W once and X chunks through a 4-stage ring
-// with TMA (128-byte swizzle); warp 1 issues the MMAs from one thread; warps
-// 4..19 are the epilogue (warp w reads TMEM lanes 32 (w % 4) .. +31, i.e. chains,
-// and a quarter of the columns).  All waits are bounded: on expiry the CTA records
+// with TMA (128-byte swizzle); warps 1 and 2 issue the Z and the G products; warps
+// 4..19 are the epilogue, in two groups that take alternate chunks (one group's waits
+// for Z and its tensor-memory loads overlap the other's arithmetic); warp w reads TMEM
+// lanes 32 (w % 4) .. +31, i.e. chains, and half of the columns.  All waits are bounded: on expiry the CTA records
 // ST_TIMEOUT in the status word, drains what it issued and frees its tensor memory.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -52,7 +54,7 @@ constexpr int TNR = 128;     // data rows per chunk (MMA N of Z, K of G)
 constexpr int NSTAGE = 4;    // X ring depth
 constexpr int NTHR = 640;
 constexpr int EPI_WARP0 = 4;  // first epilogue warp
-constexpr int NEPI = 16;      // epilogue warps: 4 lane quarters x 4 column quarters
+constexpr int NEPI = 16;      // epilogue warps: 2 groups (even and odd chunks) x 2 column halves x 4 lane quarters
 
 using namespace tc;
 
@@ -114,7 +116,7 @@ struct Smem {
 
 enum { B_WFULL = 0, B_XFULL = 1, B_XEMPTY = B_XFULL + NSTAGE, B_ZFULL = B_XEMPTY + NSTAGE,
        B_ZEMPTY = B_ZFULL + 2, B_RFULL = B_ZEMPTY + 2, B_REMPTY = B_RFULL + 2,
-       B_GDONE = B_REMPTY + 2, B_DRAIN = B_GDONE + 1, NBAR = B_DRAIN + 1 };
+       B_GDONE = B_REMPTY + 2, B_DRAIN = B_GDONE + 1, NBAR = B_DRAIN + 2 };
 
 template <int KP, bool FOLD>
 __global__ void __launch_bounds__(NTHR, 1)
@@ -133,7 +135,7 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
     ff* s_lp = reinterpret_cast<ff*>(gbase + S::OFF_LP);
     auto bar = [&](int k) { return bars + 8u * (uint32_t)k; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int64_t m0 = (int64_t)blockIdx.x * MT;
     const int split = blockIdx.y;
     const int r_begin = split * A.rps;
@@ -149,12 +151,13 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar(B_ZFULL + b), 1);
-            mbar_init(bar(B_ZEMPTY + b), NEPI);
-            mbar_init(bar(B_RFULL + b), NEPI);
+            mbar_init(bar(B_ZEMPTY + b), NEPI / 2);
+            mbar_init(bar(B_RFULL + b), NEPI / 2);
             mbar_init(bar(B_REMPTY + b), 1);
         }
         mbar_init(bar(B_GDONE), 1);
         mbar_init(bar(B_DRAIN), 1);
+        mbar_init(bar(B_DRAIN + 1), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_fail = 0;
     }
@@ -167,7 +170,7 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = s_tmem;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
     const uint32_t tZ = tmem, tG = tmem + 2 * TNR, tR = tmem + S::T_R;
 
     if (warp == 0) {
@@ -198,82 +201,99 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
         }
       }
       __syncwarp();
-    } else if (warp == 1) {
-      if (lane == 0) {
-        // ------------------------------------------------ MMA issuer
-        constexpr uint32_t ID_Z = idesc_bf16(MT, TNR);
+    } else if (warp <= 2) {
+        // ------------------------------------------------ MMA issuers: warp 1 Z, warp 2 G
+        // (the whole warp runs the loop, one elected lane issues).  A warp each, so that the
+        // waits, fences and commits of one chain do not hold up the other's products: with one
+        // thread for both, the tensor pipe stood idle for 40% of each chunk's 1344 clocks.
         const int k16 = (A.d + 15) / 16;  // K steps of one term of Z; N of G
-        const uint32_t ID_G = idesc_bf16(MT, 16 * k16, true);
-        const uint64_t dX = sw128_desc(sX), dXmn = sw128_mn_desc(sX, S::ATOM), dW = sw128_desc(sW);
-        bool ok = mbar_wait(bar(B_WFULL), 0, deadline);
-        tc_fence_after();
-        auto gemm2 = [&](int cc) -> bool {
-            const int rb = cc & 1, st = cc % NSTAGE;
-            if (!mbar_wait(bar(B_RFULL + rb), (cc >> 1) & 1, deadline)) return false;
-            tc_fence_after();
-            const uint32_t aR = tR + (uint32_t)rb * (TNR / 2);
-            const uint64_t bX = dXmn + (uint64_t)((uint32_t)st * S::STAGE >> 4);
-#pragma unroll
-            for (int kk = 0; kk < TNR / 16; ++kk)
-                tc_mma_ts(tG, aR + 8u * kk, bX + (2048u * kk >> 4), ID_G, (cc > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(bar(B_REMPTY + rb));
-            tc_commit(bar(B_XEMPTY + st));
-            return true;
-        };
-        for (int c = 0; c <= nc && ok; ++c) {
-            if (c < nc) {
+        bool ok = true;
+        if (warp == 1) {
+            constexpr uint32_t ID_Z = idesc_bf16(MT, TNR);
+            const uint64_t dX = sw128_desc(sX), dW = sw128_desc(sW);
+            ok = __all_sync(0xffffffffu, mbar_wait(bar(B_WFULL), 0, deadline));
+            for (int c = 0; c < nc && ok; ++c) {
                 const int st = c % NSTAGE, zb = c & 1;
-                if (!mbar_wait(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) ||
-                    !mbar_wait(bar(B_ZEMPTY + zb), ((c >> 1) & 1) ^ 1, deadline)) {
-                    ok = false;
-                    break;
-                }
+                ok = mbar_wait(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) &&
+                     mbar_wait(bar(B_ZEMPTY + zb), ((c >> 1) & 1) ^ 1, deadline);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
                 tc_fence_after();
                 const uint64_t bX = dX + (uint64_t)((uint32_t)st * S::STAGE >> 4);
                 const uint32_t dZ = tZ + (uint32_t)zb * TNR;
+                if (elect_one()) {
 #pragma unroll
-                for (int part = 0; part < 2; ++part)
+                    for (int part = 0; part < 2; ++part)
 #pragma unroll
-                    for (int kk = 0; kk < KP / 16; ++kk)
-                        if (kk < k16)
-                            tc_mma(dZ, dW + (((uint32_t)(part * S::NA + kk / 4) * (MT * 128) + 32u * (kk % 4)) >> 4),
-                                   bX + (((uint32_t)(kk / 4) * S::ATOM + 32u * (kk % 4)) >> 4), ID_Z,
-                                   part + kk > 0 ? 1u : 0u);
-                tc_commit(bar(B_ZFULL + zb));
+                        for (int kk = 0; kk < KP / 16; ++kk)
+                            if (kk < k16)
+                                tc_mma(dZ, dW + (((uint32_t)(part * S::NA + kk / 4) * (MT * 128) + 32u * (kk % 4)) >> 4),
+                                       bX + (((uint32_t)(kk / 4) * S::ATOM + 32u * (kk % 4)) >> 4), ID_Z,
+                                       part + kk > 0 ? 1u : 0u);
+                    tc_commit(bar(B_ZFULL + zb));
+                }
+                __syncwarp();
             }
-            if (c >= 1 && !gemm2(c - 1)) { ok = false; break; }
-        }
-        if (ok) {
-            tc_commit(bar(B_GDONE));
         } else {
-            atomicExch(&s_fail, 1);
-            tc_commit(bar(B_DRAIN));  // everything issued so far has completed once this arrives
-            mbar_wait(bar(B_DRAIN), 0, global_ns() + drain_ns(A.timeout_ns));
+            const uint32_t ID_G = idesc_bf16(MT, 16 * k16, true);
+            const uint64_t dXmn = sw128_mn_desc(sX, S::ATOM);
+            for (int c = 0; c < nc && ok; ++c) {
+                const int rb = c & 1, st = c % NSTAGE;
+                ok = mbar_wait(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) &&
+                     mbar_wait(bar(B_RFULL + rb), (c >> 1) & 1, deadline);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t aR = tR + (uint32_t)rb * (TNR / 2);
+                const uint64_t bX = dXmn + (uint64_t)((uint32_t)st * S::STAGE >> 4);
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < TNR / 16; ++kk)
+                        tc_mma_ts(tG, aR + 8u * kk, bX + (2048u * kk >> 4), ID_G, (c > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(bar(B_REMPTY + rb));
+                    tc_commit(bar(B_XEMPTY + st));
+                    if (c == nc - 1) tc_commit(bar(B_GDONE));
+                }
+                __syncwarp();
+            }
+            if (nc == 0 && elect_one()) mbar_arrive(bar(B_GDONE));
         }
-      }
-      __syncwarp();
+        if (!ok) {
+            if (elect_one()) {
+                atomicExch(&s_fail, 1);
+                tc_commit(bar(B_DRAIN + warp - 1));  // everything this warp issued has completed once it arrives
+                mbar_wait(bar(B_DRAIN + warp - 1), 0, global_ns() + drain_ns(A.timeout_ns));
+            }
+            __syncwarp();
+        }
     } else if (warp >= EPI_WARP0 && warp < EPI_WARP0 + NEPI) {
         // ------------------------------------------------ epilogue
         const int q = warp & 3;                 // TMEM lane quarter: chains 32q .. 32q+31
-        constexpr int ZC = TNR / 4;             // Z columns of one warp
-        const int h = (warp - EPI_WARP0) >> 2;  // column quarter: Z columns ZC h .. ZC h + ZC - 1
+        constexpr int ZC = 32;                  // Z columns of one pass (two passes a warp)
+        const int h = (warp - EPI_WARP0) >> 2;
+        const int grp = h >> 1, half = h & 1;   // chunks c = grp (mod 2); Z columns 64 half .. + 63
         const int rt = 32 * q + lane;           // this thread's chain in the tile
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
         const f32x2 one2 = pack2(1.0f, 1.0f), m1 = pack2(-1.0f, -1.0f);
         const f32x2 nln2 = pack2(-0.6931471805599453f, -0.6931471805599453f);
         ff lp = ff_make(0.0f);
         bool ok = true;
-        for (int c = 0; c < nc; ++c) {
-            const int zb = c & 1;
-            const int row0 = r_begin + c * TNR + ZC * h;
-            const int nlive = min(ZC, max(0, r_end - row0));
+        for (int c = grp; c < nc && ok; c += 2) {
+            const int zb = grp, rb = grp;  // Z and R buffers of this group
             if (!mbar_wait(bar(B_ZFULL + zb), (c >> 1) & 1, deadline)) { ok = false; break; }
             tc_fence_after();
+#pragma unroll
+            for (int pass = 0; pass < 2; ++pass) {
+            const int col0 = 64 * half + ZC * pass;
+            const int row0 = r_begin + c * TNR + col0;
+            const int nlive = min(ZC, max(0, r_end - row0));
             float z[ZC];
-            tmem_ld32(tZ + lane_off + (uint32_t)(zb * TNR + ZC * h), z);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_ZEMPTY + zb));
+            tmem_ld32(tZ + lane_off + (uint32_t)(zb * TNR + col0), z);
+            if (pass == 1) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_ZEMPTY + zb));
+            }
             // Fast SFU approximations (this form serves the unadjusted phase only):
             // t = e^{-|z|}, sigmoid = (z >= 0 ? 1 : t) / (1 + t), softplus = max(z, 0) +
             // log(1 + t)
@@ -340,10 +360,11 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
                 const float2 ls = unpack2(lsum);
                 lp = ff_add(ff_add(lp, ls.x), ls.y);
             }
-            const int rb = zb;
-            if (!mbar_wait(bar(B_REMPTY + rb), ((c >> 1) & 1) ^ 1, deadline)) { ok = false; break; }
-            // R row rt, data rows ZC h .. ZC h + ZC - 1: columns ZC/2 h .. of this lane's R buffer
-            tmem_st16(tR + lane_off + (uint32_t)(rb * (TNR / 2) + (ZC / 2) * h), pr);
+            if (pass == 0 && !mbar_wait(bar(B_REMPTY + rb), ((c >> 1) & 1) ^ 1, deadline)) { ok = false; break; }
+            // R row rt, data rows col0 .. col0 + 31 of the chunk: columns col0 / 2 .. of this lane's R buffer
+            tmem_st16(tR + lane_off + (uint32_t)(rb * (TNR / 2) + col0 / 2), pr);
+            }
+            if (!ok) break;
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
