@@ -461,56 +461,28 @@ __global__ void __launch_bounds__(kMaxThreads) laps_resident_kernel(const KParam
         }
         LAPS_PHASE_MARK(1);
         // ------------------------------------------------ 2. block columns
-        const int nq = ens_nq(P, H);
-        if (nq == NQ && P.qpp >= NQ) {
-            // all four quantities in one pass (the usual case): y, y^2, g, y g of each
-            // coordinate formed together; the same values and summation order as below
+        if (gl == 0) {
+            float* cs = s_cs + (size_t)slot * NCSF;
+            cs[0] = c_d.hi; cs[1] = c_d.lo; cs[2] = c_d2; cs[3] = c_fin; cs[4] = c_bad; cs[5] = c_a;
+        }
+        // one quantity of the warp's chains into its shared row: the warp's groups by
+        // shuffles, a coordinate block per 16-byte store
+        auto put_row = [&](float* row, int k, const float (&v)[4]) {
+            const int j = gl + LPC * k;
+            float4 t;
+            float* tv = &t.x;
 #pragma unroll
-            for (int k = 0; k < NB; ++k) {
-                const int j = gl + LPC * k;
+            for (int c = 0; c < 4; ++c) tv[c] = across_groups<LPC>(active ? v[c] : 0.0f);
+            if (grp == 0 && j < P.nblk) *reinterpret_cast<float4*>(row + 4 * j) = t;
+        };
+        auto quantity = [&](int qd, int k, float (&v)[4]) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int q = 4 * k + c;
-                    const float yv = active ? y[q] : 0.0f, gv = active ? g[q] : 0.0f;
-                    const float v0 = across_groups<LPC>(yv), v1 = across_groups<LPC>(yv * yv);
-                    const float v2 = across_groups<LPC>(gv), v3 = across_groups<LPC>(yv * gv);
-                    if (grp == 0 && j < P.nblk) {
-                        float* row = sq + (size_t)warp * dp + 4 * j + c;
-                        row[0] = v0;
-                        row[(size_t)nwarps * dp] = v1;
-                        row[(size_t)2 * nwarps * dp] = v2;
-                        row[(size_t)3 * nwarps * dp] = v3;
-                    }
-                }
+            for (int c = 0; c < 4; ++c) {
+                const int q = 4 * k + c;
+                v[c] = qd == 0 ? y[q] : qd == 1 ? y[q] * y[q] : qd == 2 ? g[q] : y[q] * g[q];
             }
-            __syncthreads();
-            for (int col = tid; col < NQ * dp; col += blockDim.x) {
-                const int qd = col / dp, i = col - qd * dp;
-                if (i >= P.d) continue;
-                ff s = ff_make(0.0f);
-                const float* src = sq + (size_t)qd * nwarps * dp + i;
-                for (int w = 0; w < nwarps; ++w) s = ff_add(s, src[(size_t)w * dp]);
-                P.part[((size_t)qd * dp + i) * G + blockIdx.x] = make_float2(s.hi, s.lo);
-            }
-            __syncthreads();
-        } else
-        for (int q0 = 0; q0 < nq; q0 += P.qpp) {
-            const int q1 = min(nq, q0 + P.qpp);
-            for (int qd = q0; qd < q1; ++qd) {
-#pragma unroll
-                for (int k = 0; k < NB; ++k) {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int q = 4 * k + c;
-                        float v = qd == 0 ? y[q] : qd == 1 ? y[q] * y[q] : qd == 2 ? g[q] : y[q] * g[q];
-                        v = active ? v : 0.0f;
-                        v = across_groups<LPC>(v);
-                        const int j = gl + LPC * k;
-                        if (grp == 0 && j < P.nblk) sq[((size_t)(qd - q0) * nwarps + warp) * dp + 4 * j + c] = v;
-                    }
-                }
-            }
-            __syncthreads();
+        };
+        auto add_columns = [&](int q0, int q1) {
             for (int col = tid; col < (q1 - q0) * dp; col += blockDim.x) {
                 const int qd = q0 + col / dp, i = col - (col / dp) * dp;
                 if (i >= P.d) continue;
@@ -519,16 +491,38 @@ __global__ void __launch_bounds__(kMaxThreads) laps_resident_kernel(const KParam
                 for (int w = 0; w < nwarps; ++w) s = ff_add(s, src[(size_t)w * dp]);
                 P.part[((size_t)qd * dp + i) * G + blockIdx.x] = make_float2(s.hi, s.lo);
             }
+        };
+        const int nq = ens_nq(P, H);
+        if (nq == NQ && P.qpp >= NQ) {
+            // all four quantities in one pass (the usual case)
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+#pragma unroll
+                for (int qd = 0; qd < NQ; ++qd) {
+                    float v[4];
+                    quantity(qd, k, v);
+                    put_row(sq + ((size_t)qd * nwarps + warp) * dp, k, v);
+                }
             __syncthreads();
+            add_columns(0, NQ);
+        } else
+        for (int q0 = 0; q0 < nq; q0 += P.qpp) {
+            const int q1 = min(nq, q0 + P.qpp);
+            if (q0 > 0) __syncthreads();  // the previous pass's rows are consumed
+            for (int qd = q0; qd < q1; ++qd)
+#pragma unroll
+                for (int k = 0; k < NB; ++k) {
+                    float v[4];
+                    quantity(qd, k, v);
+                    put_row(sq + ((size_t)(qd - q0) * nwarps + warp) * dp, k, v);
+                }
+            __syncthreads();
+            add_columns(q0, q1);
         }
         LAPS_PHASE_MARK(2);
-        if (gl == 0) {
-            float* cs = s_cs + (size_t)slot * NCSF;
-            cs[0] = c_d.hi; cs[1] = c_d.lo; cs[2] = c_d2; cs[3] = c_fin; cs[4] = c_bad; cs[5] = c_a;
-        }
-        __syncthreads();
-        // per-chain sums: warp k adds quantity k over the slots (lanes, then a butterfly)
-        for (int k = warp; k < NCS; k += nwarps) {
+        // per-chain sums, beside the columns: the last warps (which have the fewest columns)
+        // add one quantity each over the slots (lanes, then a butterfly)
+        for (int k = nwarps - 1 - warp; k < NCS; k += nwarps) {
             ff s = ff_make(0.0f);
             for (int sl = lane; sl < slots; sl += 32) {
                 const float* cs = s_cs + (size_t)sl * NCSF;
