@@ -427,8 +427,6 @@ laps_status laps_target_create(const laps_target_desc* desc, laps_target** out) 
         if (logreg_mma_supported(L.kp) && logreg_mma_prepare(L) != cudaSuccess) {
             cudaGetLastError();
             if (L.Xb) cudaFree(L.Xb);
-            if (L.Xf) cudaFree(L.Xf);
-            if (L.yp) cudaFree(L.yp);
             L.Xb = L.Xf = nullptr;
             L.yp = nullptr;
         }
@@ -455,8 +453,6 @@ void laps_target_destroy(laps_target* t) {
     if (t->lr.X) cudaFree(t->lr.X);
     if (t->lr.y) cudaFree(t->lr.y);
     if (t->lr.Xb) cudaFree(t->lr.Xb);
-    if (t->lr.Xf) cudaFree(t->lr.Xf);
-    if (t->lr.yp) cudaFree(t->lr.yp);
     if (t->lr.X3b) cudaFree(t->lr.X3b);
     if (t->status) cudaFree(t->status);
     delete t;

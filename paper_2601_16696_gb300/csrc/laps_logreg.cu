@@ -391,49 +391,57 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     }
 }
 
-// kp <= 128: the packed kernel (its accumulators and Z tile need 250 registers at
-// kp = 192 and above, where the plain kernel keeps its 4 x 4 tiles)
+// kp <= 128 has the packed kernel (its accumulators and Z tile need 250 registers at
+// kp = 192 and above).  It takes the launch when some SM gets two blocks; below that an
+// SM holds one block, whose four warps reach 83 of the FMA pipe's 128 lanes a clock, and the
+// plain kernel's eight are faster (n = 262, d = 72, M = 198, 20 blocks: 15 steps of a run
+// 787 against 847 us).  Both give the same bits.
 template <int KP>
 constexpr bool kPacked = KP <= 128;
 
 template <int KP>
-size_t f32_smem() {
+size_t f32_smem(bool packed) {
     const size_t tiles = (size_t)TM * (KP + 4) + (size_t)TN * (KP + 4) + TM;
-    if (kPacked<KP>) return (tiles + (size_t)TN * RTP + 2 * TM) * sizeof(float);  // W: TM / 2 rows of 2 kp + 4
+    if (packed) return (tiles + (size_t)TN * RTP + 2 * TM) * sizeof(float);  // W: TM / 2 rows of 2 kp + 4
     return (tiles + (size_t)TN * RTS) * sizeof(float);
-}
-
-template <int KP>
-const void* f32_fn() {
-    if constexpr (kPacked<KP>) return (const void*)logreg_grad_f32p_kernel<KP>;
-    else return (const void*)logreg_grad_f32_kernel<KP>;
 }
 
 template <int KP>
 cudaError_t launch_f32(const LogregData& D, const float* W, int64_t M, int S, float* gpart,
                        float2* lpart, cudaStream_t st, const int* guard) {
-    const size_t smem = f32_smem<KP>();
-    cudaError_t e = cudaFuncSetAttribute(f32_fn<KP>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     const int rps = (D.n + S - 1) / S;
     const dim3 grid((unsigned)((M + TM - 1) / TM), (unsigned)S);
-    if constexpr (kPacked<KP>)
-        logreg_grad_f32p_kernel<KP><<<grid, PT, smem, st>>>(W, M, D.X, D.y, D.n, (D.d + 3) / 4 * 4, rps, D.inv_v, gpart,
-                                                            lpart, guard);
-    else
-        logreg_grad_f32_kernel<KP><<<grid, NT, smem, st>>>(W, M, D.X, D.y, D.n, rps, D.inv_v, gpart, lpart, guard);
+    if constexpr (kPacked<KP>) {
+        int dev = 0, nsm = 1;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if ((int64_t)grid.x * S > nsm) {
+            const size_t smem = f32_smem<KP>(true);
+            e = cudaFuncSetAttribute(logreg_grad_f32p_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            logreg_grad_f32p_kernel<KP><<<grid, PT, smem, st>>>(W, M, D.X, D.y, D.n, (D.d + 3) / 4 * 4, rps, D.inv_v,
+                                                                gpart, lpart, guard);
+            return cudaGetLastError();
+        }
+    }
+    const size_t smem = f32_smem<KP>(false);
+    cudaError_t e = cudaFuncSetAttribute(logreg_grad_f32_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    logreg_grad_f32_kernel<KP><<<grid, NT, smem, st>>>(W, M, D.X, D.y, D.n, rps, D.inv_v, gpart, lpart, guard);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 namespace {
+// blocks per SM the data split plans for: the plain kernel's (the packed one's is the same)
 template <int KP>
 int f32_blocks_per_sm() {
     int n = 0;
-    if (cudaFuncSetAttribute(f32_fn<KP>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f32_smem<KP>()) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f32_fn<KP>(), kPacked<KP> ? PT : NT, f32_smem<KP>()) !=
+    if (cudaFuncSetAttribute(logreg_grad_f32_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)f32_smem<KP>(false)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, logreg_grad_f32_kernel<KP>, NT, f32_smem<KP>(false)) !=
             cudaSuccess) {
         cudaGetLastError();
         n = 0;

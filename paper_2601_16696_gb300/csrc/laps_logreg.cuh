@@ -21,7 +21,7 @@ struct LogregData {
     float* y;         // [n] labels
     float inv_v;      // 1 / prior variance
     // tensor-core form (kp <= 128): BF16 copies and their TMA descriptors
-    void* Xb;         // [n][kp] BF16
+    void* Xb;         // [n][kp] BF16 (owns Xf and yp, in the same allocation)
     void* Xf;         // the same with the rows of label 1 negated
     float* yp;        // [n rounded up to 32] labels in pairs of rows (j, j + 16) of each 32
     bool bin;         // every label is 0 or 1
@@ -38,7 +38,7 @@ constexpr int kLogregMaxKp = 256;
 
 // ---- tensor-core (tcgen05, BF16) gradient: laps_logreg_mma.cu
 bool logreg_mma_supported(int kp);
-// BF16 copies of X, their tensor maps and the paired labels (allocates Xb, Xf, yp; synchronises)
+// BF16 copies of X, their tensor maps and the paired labels (allocates Xb; synchronises)
 cudaError_t logreg_mma_prepare(LogregData& D);
 // tensor map of the [M_pad][2 kp] BF16 (hi | lo) copy of the points
 cudaError_t logreg_mma_wmap(void* tmW, const void* Wb, int64_t M_pad, int kp);

@@ -497,14 +497,14 @@ cudaError_t logreg_mma_prepare(LogregData& D) {
     if (!logreg_mma_supported(D.kp)) return cudaErrorInvalidValue;
     EncodeTiled enc = encoder();
     if (!enc) return cudaErrorNotSupported;
+    // one allocation: Xb, Xf, the paired labels, the flag of other labels
     const size_t nb = (size_t)D.n * D.kp * sizeof(__nv_bfloat16);
     const int n32 = (D.n + 31) / 32 * 32;
-    int* other = nullptr;
-    cudaError_t e = cudaMalloc(&D.Xb, nb);
-    if (e == cudaSuccess) e = cudaMalloc(&D.Xf, nb);
-    if (e == cudaSuccess) e = cudaMalloc(&D.yp, (size_t)n32 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&other, sizeof(int));
+    cudaError_t e = cudaMalloc(&D.Xb, 2 * nb + (size_t)n32 * sizeof(float) + sizeof(int));
     if (e != cudaSuccess) return e;
+    D.Xf = static_cast<char*>(D.Xb) + nb;
+    D.yp = reinterpret_cast<float*>(static_cast<char*>(D.Xb) + 2 * nb);
+    int* other = reinterpret_cast<int*>(D.yp + n32);
     int h_other = 0;
     e = cudaMemset(other, 0, sizeof(int));
     if (e == cudaSuccess) {
@@ -514,14 +514,13 @@ cudaError_t logreg_mma_prepare(LogregData& D) {
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(&h_other, other, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaFree(other);
     if (e != cudaSuccess) return e;
     D.bin = h_other == 0;
     // [n][kp], boxes of 64 features x 128 rows (rows past n read as zero)
     if (!encode_bf16_2d(D.tmX, D.Xb, (uint64_t)D.kp, (uint64_t)D.n, 64, TNR) ||
         !encode_bf16_2d(D.tmXf, D.Xf, (uint64_t)D.kp, (uint64_t)D.n, 64, TNR))
         return cudaErrorInvalidValue;
-    return cudaDeviceSynchronize();
+    return cudaSuccess;  // the copy of the flag waited for both kernels
 }
 
 cudaError_t logreg_mma_wmap(void* tmW, const void* Wb, int64_t M_pad, int kp) {
