@@ -188,9 +188,10 @@ laps_status choose_shape(laps_ctx* c) {
     // Among the block sizes of that lane shape, 256 threads while the blocks still fit one per
     // SM: the chain updates, the reductions' slices and the per-block columns then spread over
     // twice the SMs; the lane shape stays, so does every chain's arithmetic.  Measured, us per
-    // unadjusted iteration / per proposal at 512 -> 256 threads: d = 100, M = 256 11.8 / 66 ->
-    // 12.4 / 47; M = 1024 12.6 / 66 -> 11.5 / 48; d = 10, M = 256 9.2 / 41 -> 7.7 / 29; d = 300,
-    // M = 512 22.1 / 162 -> 19.7 / 127.  128 threads: 15.5 / 43, 12.8 / 42, 8.7 / 27, 21.3 / 113.
+    // unadjusted iteration / per proposal, 512 against 256 threads: d = 100, M = 1024 12.6 / 66
+    // against 10.7 / 46; M = 256 11.8 / 66 against 11.0 / 46; d = 10, M = 256 9.2 / 41 against
+    // 8.6 / 29; d = 300, M = 1000 21.6 / 162 against 18.5 / 125.  128 threads gain a tenth of a
+    // proposal and lose a tenth of an unadjusted iteration.
     if (c->cfg.chains_per_block == 0 && c->cfg.dtilde_K == 0)
         for (int k = 0; k < n_ok; ++k)
             if (ok[k].lpc == best.lpc && ok[k].cpl == best.cpl && ok[k].threads == 256 && best.threads > 256 &&

@@ -653,9 +653,7 @@ __global__ void __launch_bounds__(kBT, 1) batch_kernel(const __grid_constant__ B
         if (!grid_sync_count(B.bar_count, B.status, n_bar * (unsigned)(G + B.bar_extra), B.timeout_ns)) return;
         for (int p = b; p < B.n; p += G) {
             load_prob(p);
-            const bool skip = B.mode == 1 && sH.done;
-            __syncthreads();  // every thread has read the phase machine before the finalise updates it
-            if (skip) continue;
+            if (B.mode == 1 && sH.done) continue;
             ens_gather(sP, sH, qbuf, FS);
             if (tid == 0) {
                 *sP.hyper = sH;

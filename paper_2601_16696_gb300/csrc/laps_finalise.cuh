@@ -69,16 +69,7 @@ __device__ __forceinline__ void ens_slice(const KParams& P, const Hyper& H, ff* 
     const int ns = i1 - i0;
     const bool push = (P.mode == 1 && H.phase == 0);
     const int win_n = H.win_n;
-    // Per coordinate three results that need only the column sums: the variances and
-    // (1 - V)^2, the window statistic, b^2.  Each is a serial chain of float-float
-    // operations, so they go to different warps: item idx is role idx / nsr of
-    // coordinate idx % nsr.  (One thread per coordinate ran them one after another; with
-    // the sums below and the smaller gather, d = 100, M = 32 takes 11.7 us per unadjusted
-    // iteration in place of 35, M = 256 12.4 in place of 14.7, banana M = 4096 12.9 in place
-    // of 13.3.)
-    const int nsr = (ns + 31) & ~31;
-    const int role = tid < nsr ? 0 : tid < 2 * nsr ? 1 : 2, k_own = tid - role * nsr;
-    // the values this thread's first item needs, loaded before the reductions
+    // the window values this thread will update, loaded before the reductions
     float4 w_pre = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     float2 o_pre = make_float2(0.0f, 0.0f), e_pre = make_float2(0.0f, 0.0f);
     float sg_pre = 1.0f, pr_pre = 0.0f, iv_pre = 0.0f;
@@ -86,113 +77,113 @@ __device__ __forceinline__ void ens_slice(const KParams& P, const Hyper& H, ff* 
     // kept before this slice replaces them with the current means
     const bool fr_live = P.dfull_K > 0 && s_fr != nullptr;
     float* s_old = fr_live ? reinterpret_cast<float*>(s_fr + 2 * blockDim.x) : nullptr;  // [ns]
-    if (k_own < ns && tid < 3 * nsr) {
-        const int i = i0 + k_own;
+    if (tid < ns) {
+        const int i = i0 + tid;
+        if (fr_live) s_old[tid] = __ldcg(P.cstat + (size_t)i * NCO + CO_MY);
+        if (push) {
+            w_pre = P.win_sums[i];
+            if (win_n >= P.T) o_pre = P.ring[(size_t)((win_n - P.T) % (P.T + 1)) * dp + i];
+        }
         sg_pre = P.sigma[i];
-        if (role == 0) {
-            if (P.gauss_derived) pr_pre = P.prec[i];
-        } else if (role == 1) {
-            if (push) {
-                w_pre = P.win_sums[i];
-                if (win_n >= P.T) o_pre = P.ring[(size_t)((win_n - P.T) % (P.T + 1)) * dp + i];
-            }
-        } else if (P.Ex2) {
+        if (P.gauss_derived) pr_pre = P.prec[i];
+        if (P.Ex2) {
             e_pre = P.Ex2[i];
             iv_pre = P.inv_varx2[i];
         }
     }
-    if (fr_live && tid < ns) s_old[tid] = __ldcg(P.cstat + (size_t)(i0 + tid) * NCO + CO_MY);
-    // column sums over the blocks, in block order: a warp per (quantity, coordinate), or
-    // with fewer than 32 blocks several per warp (the same butterfly without its zeros)
+    // column sums over the blocks, in block order: one warp per (quantity, coordinate), or
+    // with fewer than 32 blocks (and so longer slices) several per warp: the same butterfly
+    // without its zeros (d = 10, M = 256, 4 blocks: 10.5 -> 8.6 us per unadjusted iteration).
+    // The code below and the finalise run once an iteration on few warps, where what counts
+    // is how little of it there is to fetch: splitting a coordinate's results over three
+    // warps and unrolling the gather for one warp made the iteration slower.
     const int n_pairs = nq * ns + (chain_owner ? NCS : 0);
-    const int lpp = G >= 32 ? 32 : G <= 1 ? 1 : 1 << (32 - __clz(G - 1));
-    const int ppw = 32 / lpp, sub = lane / lpp, sl = lane - sub * lpp;
-    for (int p0 = warp * ppw; p0 < n_pairs; p0 += nwarps * ppw) {
-        const int pidx = p0 + sub;
-        ff s = ff_make(0.0f);
-        if (pidx < n_pairs) {
-            size_t row;
-            if (pidx < nq * ns) row = (size_t)(pidx / ns) * dp + i0 + (pidx % ns);
-            else row = (size_t)NQ * dp + (pidx - nq * ns);
-            s = lane_col_sum(P.part + row * G, G, sl, lpp);
+    auto row_of = [&](int pidx) {
+        return pidx < nq * ns ? (size_t)(pidx / ns) * dp + i0 + (pidx % ns) : (size_t)NQ * dp + (pidx - nq * ns);
+    };
+    auto put = [&](int pidx, ff s) {
+        if (pidx < nq * ns) s_q[(pidx / ns) * P.smax + (pidx % ns)] = s;
+        else s_q[NQ * P.smax + (pidx - nq * ns)] = s;
+    };
+    if (G >= 32) {
+        for (int pidx = warp; pidx < n_pairs; pidx += nwarps) {
+            ff s = lane_col_sum(P.part + row_of(pidx) * G, G, lane, 32);
+            s = group_sum_ff<32>(s);
+            if (lane == 0) put(pidx, s);
         }
-        for (int o = lpp / 2; o > 0; o >>= 1)
-            s = ff_add(s, ff{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
-        if (sl == 0 && pidx < n_pairs) {
-            if (pidx < nq * ns) s_q[(pidx / ns) * P.smax + (pidx % ns)] = s;
-            else s_q[NQ * P.smax + (pidx - nq * ns)] = s;
+    } else {
+        const int lpp = G <= 1 ? 1 : 1 << (32 - __clz(G - 1)), ppw = 32 / lpp, sub = lane / lpp, sl = lane - sub * lpp;
+        for (int p0 = warp * ppw; p0 < n_pairs; p0 += nwarps * ppw) {
+            const int pidx = p0 + sub;
+            ff s = ff_make(0.0f);
+            if (pidx < n_pairs && sl < G) {
+                const float2 v = __ldcg(P.part + row_of(pidx) * G + sl);
+                s = ff{v.x, v.y};
+            }
+            for (int o = lpp / 2; o > 0; o >>= 1)
+                s = ff_add(s, ff{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
+            if (sl == 0 && pidx < n_pairs) put(pidx, s);
         }
     }
     __syncthreads();
     const float iM = 1.0f / (float)ens_chains(P);
-    for (int idx = tid; idx < 3 * nsr; idx += blockDim.x) {
-        const int r = idx < nsr ? 0 : idx < 2 * nsr ? 1 : 2, k = idx - r * nsr;
-        if (k >= ns) continue;
-        const bool own = idx == tid;
+    for (int k = tid; k < ns; k += blockDim.x) {
         const int i = i0 + k;
-        float* co = P.cstat + (size_t)i * NCO;
+        const ff mean = ff_mulf(s_q[0 * P.smax + k], iM);
         const ff ey2 = ff_mulf(s_q[1 * P.smax + k], iM);
-        const float sgi = own ? sg_pre : P.sigma[i];
+        const float var_y = ff_f(ff_add(ey2, ff_neg(ff_mul(mean, mean))));
+        const float sgi = k == tid ? sg_pre : P.sigma[i];
         const float s2i = sgi * sgi;
-        if (r == 0) {
-            const ff mean = ff_mulf(s_q[0 * P.smax + k], iM);
-            const float var_y = ff_f(ff_add(ey2, ff_neg(ff_mul(mean, mean))));
-            float dv = 0.0f;
-            if (nq == NQ) {
-                // V_ii = -(E[y g] - E[y] E[g])  (App. B, Eq. ECA)
-                const ff eg = ff_mulf(s_q[2 * P.smax + k], iM);
-                const ff eyg = ff_mulf(s_q[3 * P.smax + k], iM);
-                const float V = -ff_f(ff_add(eyg, ff_neg(ff_mul(mean, eg))));
-                dv = (1.0f - V) * (1.0f - V);
-            } else if (P.gauss_derived && (P.mode == 0 || H.phase == 0)) {
-                // diagonal Gaussian: g_i = -prec_i sigma_i^2 y_i, so V_ii = prec_i sigma_i^2 Var[y_i]
-                const float V = (own ? pr_pre : P.prec[i]) * s2i * var_y;
-                dv = (1.0f - V) * (1.0f - V);
-            }
-            if (fr_live) {
-                co[CO_MY] = ff_f(mean);
-                co[CO_MG] = nq == NQ ? ff_f(ff_mulf(s_q[2 * P.smax + k], iM)) : 0.0f;
-            }
-            co[CO_VARY] = var_y;
-            co[CO_VARX] = s2i * var_y;
-            co[CO_DV] = dv;
-            continue;
-        }
         const ff ex2 = ff_mulf(ey2, s2i);
-        if (r == 1) {
-            float del = 0.0f;
-            if (push) {
-                // moving window of E[x_i^2]: running sums over the last T values
-                const float4 w = own ? w_pre : P.win_sums[i];
-                ff s1{w.x, w.y}, s2{w.z, w.w};
-                float2* ring_i = P.ring + i;
-                if (win_n >= P.T) {
-                    const float2 o = own ? o_pre : ring_i[(size_t)((win_n - P.T) % (P.T + 1)) * dp];
-                    const ff old{o.x, o.y};
-                    s1 = ff_add(s1, ff_neg(old));
-                    s2 = ff_add(s2, ff_neg(ff_mul(old, old)));
-                }
-                s1 = ff_add(s1, ex2);
-                s2 = ff_add(s2, ff_mul(ex2, ex2));
-                P.win_sums[i] = make_float4(s1.hi, s1.lo, s2.hi, s2.lo);
-                ring_i[(size_t)(win_n % (P.T + 1)) * dp] = make_float2(ex2.hi, ex2.lo);
-                if (win_n + 1 >= P.T) {
-                    const float Tf = (float)P.T;
-                    const ff mu = ff_divf(s1, Tf);
-                    const float vv = ff_f(ff_add(s2, ff_neg(ff_mul(s1, mu)))) / (Tf - 1.0f);
-                    del = sqrtf(vv > 0.0f ? vv : 0.0f) / ff_f(mu);
-                }
-            }
-            co[CO_DEL] = del;
-        } else {
-            float b2 = 0.0f;
-            if (P.Ex2) {
-                const float2 e = own ? e_pre : P.Ex2[i];
-                const float dd = ff_f(ff_add(ex2, ff_neg(ff{e.x, e.y})));
-                b2 = dd * dd * (own ? iv_pre : P.inv_varx2[i]);
-            }
-            co[CO_B2] = b2;
+        float dv = 0.0f, del = 0.0f, b2 = 0.0f;
+        if (nq == NQ) {
+            // V_ii = -(E[y g] - E[y] E[g])  (App. B, Eq. ECA)
+            const ff eg = ff_mulf(s_q[2 * P.smax + k], iM);
+            const ff eyg = ff_mulf(s_q[3 * P.smax + k], iM);
+            const float V = -ff_f(ff_add(eyg, ff_neg(ff_mul(mean, eg))));
+            dv = (1.0f - V) * (1.0f - V);
+        } else if (P.gauss_derived && (P.mode == 0 || H.phase == 0)) {
+            // diagonal Gaussian: g_i = -prec_i sigma_i^2 y_i, so V_ii = prec_i sigma_i^2 Var[y_i]
+            const float V = (k == tid ? pr_pre : P.prec[i]) * s2i * var_y;
+            dv = (1.0f - V) * (1.0f - V);
         }
+        if (push) {
+            // moving window of E[x_i^2]: running sums over the last T values
+            const float4 w = k == tid ? w_pre : P.win_sums[i];
+            ff s1{w.x, w.y}, s2{w.z, w.w};
+            float2* ring_i = P.ring + i;
+            if (win_n >= P.T) {
+                const float2 o = k == tid ? o_pre : ring_i[(size_t)((win_n - P.T) % (P.T + 1)) * dp];
+                const ff old{o.x, o.y};
+                s1 = ff_add(s1, ff_neg(old));
+                s2 = ff_add(s2, ff_neg(ff_mul(old, old)));
+            }
+            s1 = ff_add(s1, ex2);
+            s2 = ff_add(s2, ff_mul(ex2, ex2));
+            P.win_sums[i] = make_float4(s1.hi, s1.lo, s2.hi, s2.lo);
+            ring_i[(size_t)(win_n % (P.T + 1)) * dp] = make_float2(ex2.hi, ex2.lo);
+            if (win_n + 1 >= P.T) {
+                const float Tf = (float)P.T;
+                const ff mu = ff_divf(s1, Tf);
+                const float vv = ff_f(ff_add(s2, ff_neg(ff_mul(s1, mu)))) / (Tf - 1.0f);
+                del = sqrtf(vv > 0.0f ? vv : 0.0f) / ff_f(mu);
+            }
+        }
+        if (P.Ex2) {
+            const float2 e = k == tid ? e_pre : P.Ex2[i];
+            const float dd = ff_f(ff_add(ex2, ff_neg(ff{e.x, e.y})));
+            b2 = dd * dd * (k == tid ? iv_pre : P.inv_varx2[i]);
+        }
+        float* co = P.cstat + (size_t)i * NCO;
+        if (fr_live) {
+            co[CO_MY] = ff_f(mean);
+            co[CO_MG] = nq == NQ ? ff_f(ff_mulf(s_q[2 * P.smax + k], iM)) : 0.0f;
+        }
+        co[CO_VARY] = var_y;
+        co[CO_VARX] = s2i * var_y;
+        co[CO_DV] = dv;
+        co[CO_DEL] = del;
+        co[CO_B2] = b2;
     }
     if (chain_owner && tid < NCS) {
         const ff v = s_q[NQ * P.smax + tid];
@@ -296,73 +287,51 @@ __device__ __forceinline__ void ens_gather(const KParams& P, Hyper& H, float* s_
     const int nwarps = blockDim.x >> 5;
     float2 tot_pre = make_float2(0.0f, 0.0f);  // warp 0, lanes < NCS: the chain totals
     if (warp == 0 && lane < NCS) tot_pre = __ldcg(P.ctot + lane);
-    // Sums over the coordinates.  Up to 256 of them warp 0 adds alone (a few per lane, one
-    // butterfly); more are spread over the block and its warps' partials combined by a
-    // second butterfly.  Both orders are fixed.
-    ff v0 = ff_make(0.0f), v1 = v0, v3 = v0, v5 = v0;  // Var x, (1 - V)^2, b^2, full-rank terms
-    float v2 = 0.0f, v4 = 0.0f;                        // maxima of delta and b^2
-    const bool full = P.dfull_K > 0 && P.mode == 1 && H.phase == 0, b2s = P.Ex2 != nullptr;
-    const bool small = P.d <= 256;
-    if (!small || warp == 0) {
-        const int step = small ? 32 : (int)blockDim.x;
-        for (int i0 = small ? lane : tid; i0 < P.d; i0 += 4 * step) {
-            float4 c4[4];
-            float cb[4], cf[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = i0 + u * step;
-                const float* co = P.cstat + (size_t)i * NCO;
-                c4[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                cb[u] = cf[u] = 0.0f;
-                if (i < P.d) {
-                    c4[u] = __ldcg(reinterpret_cast<const float4*>(co));  // Var y, Var x, (1 - V)^2, delta
-                    if (b2s) cb[u] = __ldcg(co + CO_B2);
-                    if (full) cf[u] = __ldcg(co + CO_DFULL);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = i0 + u * step;
-                if (i >= P.d) break;
-                s_var[i] = c4[u].x;
-                v0 = ff_add(v0, c4[u].y);
-                v1 = ff_add(v1, c4[u].z);
-                v2 = fmax_nan(v2, c4[u].w);
-                if (b2s) {
-                    v3 = ff_add(v3, cb[u]);
-                    v4 = fmax_nan(v4, cb[u]);
-                }
-                if (full) v5 = ff_add(v5, cf[u]);
-            }
+    {
+        ff a_var = ff_make(0.0f), a_dv = ff_make(0.0f), a_b2 = ff_make(0.0f), a_df = ff_make(0.0f);
+        float a_del = 0.0f, a_b2m = 0.0f;
+        const bool full = P.dfull_K > 0 && P.mode == 1 && H.phase == 0;
+        for (int i = tid; i < P.d; i += blockDim.x) {
+            const float* co = P.cstat + (size_t)i * NCO;
+            const float4 c4 = __ldcg(reinterpret_cast<const float4*>(co));  // Var y, Var x, (1 - V)^2, delta
+            const float vy = c4.x, vx = c4.y, dv = c4.z, del = c4.w;
+            const float b2 = P.Ex2 ? __ldcg(co + CO_B2) : 0.0f;
+            s_var[i] = vy;
+            a_var = ff_add(a_var, vx);
+            a_dv = ff_add(a_dv, dv);
+            a_b2 = ff_add(a_b2, b2);
+            if (full) a_df = ff_add(a_df, __ldcg(co + CO_DFULL));
+            a_del = fmax_nan(a_del, del);
+            a_b2m = fmax_nan(a_b2m, b2);
         }
-    }
-    auto butterfly = [&]() {
+        // one fused block reduction in a fixed order: warp butterflies, then warps in order
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            v0 = ff_add(v0, ff{__shfl_xor_sync(0xffffffffu, v0.hi, o), __shfl_xor_sync(0xffffffffu, v0.lo, o)});
-            v1 = ff_add(v1, ff{__shfl_xor_sync(0xffffffffu, v1.hi, o), __shfl_xor_sync(0xffffffffu, v1.lo, o)});
-            v2 = fmax_nan(v2, __shfl_xor_sync(0xffffffffu, v2, o));
-            if (b2s) {
-                v3 = ff_add(v3, ff{__shfl_xor_sync(0xffffffffu, v3.hi, o), __shfl_xor_sync(0xffffffffu, v3.lo, o)});
-                v4 = fmax_nan(v4, __shfl_xor_sync(0xffffffffu, v4, o));
-            }
-            if (full)
-                v5 = ff_add(v5, ff{__shfl_xor_sync(0xffffffffu, v5.hi, o), __shfl_xor_sync(0xffffffffu, v5.lo, o)});
+            const ff w0{__shfl_xor_sync(0xffffffffu, a_var.hi, o), __shfl_xor_sync(0xffffffffu, a_var.lo, o)};
+            const ff w1{__shfl_xor_sync(0xffffffffu, a_dv.hi, o), __shfl_xor_sync(0xffffffffu, a_dv.lo, o)};
+            const ff w3{__shfl_xor_sync(0xffffffffu, a_b2.hi, o), __shfl_xor_sync(0xffffffffu, a_b2.lo, o)};
+            const ff w4{__shfl_xor_sync(0xffffffffu, a_df.hi, o), __shfl_xor_sync(0xffffffffu, a_df.lo, o)};
+            a_var = ff_add(a_var, w0);
+            a_dv = ff_add(a_dv, w1);
+            a_b2 = ff_add(a_b2, w3);
+            a_df = ff_add(a_df, w4);
+            a_del = fmax_nan(a_del, __shfl_xor_sync(0xffffffffu, a_del, o));
+            a_b2m = fmax_nan(a_b2m, __shfl_xor_sync(0xffffffffu, a_b2m, o));
         }
-    };
-    if (!small) {
-        butterfly();
         if (lane == 0) {
-            FS.wsum[0][warp] = v0;
-            FS.wsum[1][warp] = v1;
-            FS.wsum[2][warp] = v3;
-            FS.wsum[3][warp] = v5;
-            FS.wmax[0][warp] = v2;
-            FS.wmax[1][warp] = v4;
+            FS.wsum[0][warp] = a_var;
+            FS.wsum[1][warp] = a_dv;
+            FS.wsum[2][warp] = a_b2;
+            FS.wsum[3][warp] = a_df;
+            FS.wmax[0][warp] = a_del;
+            FS.wmax[1][warp] = a_b2m;
         }
-        __syncthreads();
-        v0 = v1 = v3 = v5 = ff_make(0.0f);
-        v2 = v4 = 0.0f;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        // the per-warp partials combined by a butterfly over warp 0's lanes
+        ff v0 = ff_make(0.0f), v1 = v0, v3 = v0, v5 = v0;
+        float v2 = 0.0f, v4 = 0.0f;
         if (lane < nwarps) {
             v0 = FS.wsum[0][lane];
             v1 = FS.wsum[1][lane];
@@ -371,9 +340,19 @@ __device__ __forceinline__ void ens_gather(const KParams& P, Hyper& H, float* s_
             v2 = FS.wmax[0][lane];
             v4 = FS.wmax[1][lane];
         }
-    }
-    if (warp == 0) {
-        butterfly();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const ff w0{__shfl_xor_sync(0xffffffffu, v0.hi, o), __shfl_xor_sync(0xffffffffu, v0.lo, o)};
+            const ff w1{__shfl_xor_sync(0xffffffffu, v1.hi, o), __shfl_xor_sync(0xffffffffu, v1.lo, o)};
+            const ff w3{__shfl_xor_sync(0xffffffffu, v3.hi, o), __shfl_xor_sync(0xffffffffu, v3.lo, o)};
+            const ff w5{__shfl_xor_sync(0xffffffffu, v5.hi, o), __shfl_xor_sync(0xffffffffu, v5.lo, o)};
+            v0 = ff_add(v0, w0);
+            v1 = ff_add(v1, w1);
+            v3 = ff_add(v3, w3);
+            v5 = ff_add(v5, w5);
+            v2 = fmax_nan(v2, __shfl_xor_sync(0xffffffffu, v2, o));
+            v4 = fmax_nan(v4, __shfl_xor_sync(0xffffffffu, v4, o));
+        }
         ff tot[NCS];
 #pragma unroll
         for (int k = 0; k < NCS; ++k)
