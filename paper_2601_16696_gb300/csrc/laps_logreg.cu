@@ -175,7 +175,7 @@ logreg_grad_f32_kernel(const float* __restrict__ W, int64_t M, const float* __re
 
 // ---------------------------------------------------------------- packed form
 // The same contraction for kp <= 128 with packed binary32 pairs (fma.rn.f32x2),
-// every sum in the plain kernel's order (the results are its results).  What bounds
+// every sum in the plain kernel's order (the results are its results, but with ROUND).  What bounds
 // it is the FMA pipe: 2 M n d multiply-adds, of which the pipe retires 128 per clock
 // and SM either way, but a packed instruction carries two, so half the issue slots
 // are left for the operand loads and the epilogue.  A thread owns 8 chains x 4 rows
@@ -185,25 +185,32 @@ logreg_grad_f32_kernel(const float* __restrict__ W, int64_t M, const float* __re
 //      duplicated into both halves; the loop stops at the last non-zero feature
 //      (d rounded up to 4), not at the padded width;
 //   G: pairs of columns, the residual stored twice by the epilogue.
+// A target call (ROUND) rounds log p to binary32, so its log p need not be the plain
+// kernel's sum bit for bit: Z pairs even and odd k (both operands come as pairs from
+// 16-byte loads, no duplication) and the epilogue takes one log1p per four rows, of
+// prod (1 + t) - 1 built up as e <- e + t + e t (no cancellation, so small t keep their
+// relative precision; at most 15).
 // 128 threads and 64 chains per block, two blocks per SM: one block's staging and
 // epilogue overlap the other's contraction.
-// Measured at d = 101, n = 10^4, M = 8192: gradient call 1083 -> 923 us, same bits
-// (kernel 1061 -> 911 us; FMA pipe 64% busy with 23% fewer multiply-adds in Z).
+// Measured at d = 101, n = 10^4, M = 8192: gradient call 1083 -> 923 us in the plain
+// kernel's order (kernel 1061 -> 911 us; FMA pipe 64% busy with 23% fewer multiply-adds
+// in Z), 900 us with ROUND; the gradient's error against binary64 stays 2.3e-7 and
+// log p's 2.8e-8 (relative norms).
 constexpr int PT = 128;        // threads
 constexpr int RTP = 2 * TM + 4;  // row stride of the duplicated R tile
 
-template <int KP>
+template <int KP, bool ROUND>
 __global__ void __launch_bounds__(PT, 2)
 logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __restrict__ X,
                         const float* __restrict__ yv, int n, int kz, int rps, float inv_v,
                         float* __restrict__ gpart, float2* __restrict__ lpart, const int* __restrict__ guard) {
     if (guard != nullptr && *guard == 0) return;  // the iteration no longer runs
     constexpr int LD = KP + 4;       // padded row stride (floats) of the X tile
-    constexpr int LDW = 2 * KP + 4;  // and of the W tile's pairs of rows
+    constexpr int LDW = 2 * KP + 4;  // and of the W tile's pairs of rows (not ROUND)
     constexpr int NG = KP / 64;      // float4 column groups per thread in the G phase
     extern __shared__ __align__(16) float sm[];
-    float* Ws = sm;                   // [TM / 2][LDW]  row cr + 8 i: chains (cr + 16 i, cr + 16 i + 8), pairs per k
-    float* Xs = Ws + TM / 2 * LDW;    // [TN][LD]
+    float* Ws = sm;  // [TM / 2][LDW]  row cr + 8 i: chains (cr + 16 i, cr + 16 i + 8), pairs per k; ROUND: [TM][LD]
+    float* Xs = Ws + (ROUND ? TM * LD : TM / 2 * LDW);  // [TN][LD]
     float* Rt = Xs + TN * LD;         // [TN][RTP]  Rt[row][32 i + 4 cr]: chain cr + 16 i twice, cr + 16 i + 8 twice
     float* wsq = Rt + TN * RTP;       // [TM] |w|^2
     ff* s_lp = reinterpret_cast<ff*>(wsq + TM);  // [TM] log p of the upper half of the rows
@@ -214,7 +221,9 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     const int r_begin = s * rps;
     const int r_end = min(n, r_begin + rps);
     // chain r of the tile at k: row (r & 7) + 8 (r >> 4), half (r >> 3) & 1
-    auto wat = [&](int r, int k) -> float& { return Ws[((r & 7) + 8 * (r >> 4)) * LDW + 2 * k + ((r >> 3) & 1)]; };
+    auto wat = [&](int r, int k) -> float& {
+        return ROUND ? Ws[r * LD + k] : Ws[((r & 7) + 8 * (r >> 4)) * LDW + 2 * k + ((r >> 3) & 1)];
+    };
 
     // W tile (rows beyond M are zero)
     for (int k = tid; k < TM * (KP / 4); k += PT) {
@@ -249,7 +258,7 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     ff lacc[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) lacc[c] = ff_make(0.0f);
-    const float* wb = Ws + cr * LDW;
+    const float* wb = Ws + cr * (ROUND ? LD : LDW);
     const float* xb = Xs + dc * LD;
 
     for (int row0 = r_begin; row0 < r_end; row0 += TN) {
@@ -271,49 +280,72 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        // ---- Z = W X^T on the 8 x 4 thread tile, k in order
-        f32x2 z[4][4];
+        // ---- Z = W X^T on the 8 x 4 thread tile, k in order (ROUND: even and odd k apart)
+        f32x2 z[ROUND ? 8 : 4][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < (ROUND ? 8 : 4); ++i)
 #pragma unroll
             for (int e = 0; e < 4; ++e) z[i][e] = 0;
+        if constexpr (ROUND) {
 #pragma unroll 2
-        for (int k = 0; k < kz; k += 4) {
-            float4 xv[4];
+            for (int k = 0; k < kz; k += 4) {
+                ulonglong2 xv[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xv[e] = *reinterpret_cast<const float4*>(xb + 16 * e * LD + k);
+                for (int e = 0; e < 4; ++e) xv[e] = *reinterpret_cast<const ulonglong2*>(xb + 16 * e * LD + k);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                ulonglong2 wv[4];
+                for (int c = 0; c < 8; ++c) {
+                    const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(wb + 8 * c * LD + k);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) wv[i] = *reinterpret_cast<const ulonglong2*>(wb + 8 * i * LDW + 2 * k + 4 * h);
+                    for (int e = 0; e < 4; ++e) z[c][e] = fma2(wv.y, xv[e].y, fma2(wv.x, xv[e].x, z[c][e]));
+                }
+            }
+        } else {
+#pragma unroll 2
+            for (int k = 0; k < kz; k += 4) {
+                float4 xv[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float a = h == 0 ? xv[e].x : xv[e].z, b = h == 0 ? xv[e].y : xv[e].w;
-                    const f32x2 aa = pack2(a, a), bb = pack2(b, b);
+                for (int e = 0; e < 4; ++e) xv[e] = *reinterpret_cast<const float4*>(xb + 16 * e * LD + k);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) z[i][e] = fma2(wv[i].y, bb, fma2(wv[i].x, aa, z[i][e]));
+                for (int h = 0; h < 2; ++h) {
+                    ulonglong2 wv[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) wv[i] = *reinterpret_cast<const ulonglong2*>(wb + 8 * i * LDW + 2 * k + 4 * h);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float a = h == 0 ? xv[e].x : xv[e].z, b = h == 0 ? xv[e].y : xv[e].w;
+                        const f32x2 aa = pack2(a, a), bb = pack2(b, b);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) z[i][e] = fma2(wv[i].y, bb, fma2(wv[i].x, aa, z[i][e]));
+                    }
                 }
             }
         }
         // ---- epilogue: residuals and log-likelihood terms
         auto epilogue = [&](auto full) {
-            float lsum[8];
+            float lsum[8], lprod[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) lsum[c] = 0.0f;
+            for (int c = 0; c < 8; ++c) {
+                lsum[c] = 0.0f;
+                lprod[c] = 0.0f;
+            }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool ok = decltype(full)::value || row0 + dc + 16 * e < r_end;
                 float4* dst = reinterpret_cast<float4*>(Rt + (dc + 16 * e) * RTP + 4 * cr);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const float2 zp = unpack2(z[i][e]);
+                    float2 zp;
+                    if constexpr (ROUND) {
+                        const float2 za = unpack2(z[2 * i][e]), zb = unpack2(z[2 * i + 1][e]);
+                        zp = make_float2(za.x + za.y, zb.x + zb.y);
+                    } else {
+                        zp = unpack2(z[i][e]);
+                    }
                     float r[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const float zz = h == 0 ? zp.x : zp.y;
                         const float t = expf(-fabsf(zz));               // e^{-|z|} in (0, 1]
-                        const float sp = fmaxf(zz, 0.0f) + log1pf(t);   // softplus(z)
                         // 1 / (1 + t): the hardware reciprocal and two Newton steps round as the
                         // division does for every 1 + t in [1, 2] but 2 - 2^-23 (checked
                         // exhaustively from starts within two ulps)
@@ -324,13 +356,20 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
                         inv = fmaf(inv, fmaf(-opt, inv, 1.0f), inv);
                         const float sig = zz >= 0.0f ? inv : t * inv;   // sigmoid(z)
                         r[h] = ok ? yn[e] - sig : 0.0f;
-                        lsum[2 * i + h] += ok ? fmaf(yn[e], zz, -sp) : 0.0f;
+                        if constexpr (ROUND) {  // y z - max(z, 0); log(1 + t) below
+                            lsum[2 * i + h] += ok ? fmaf(yn[e], zz, -fmaxf(zz, 0.0f)) : 0.0f;
+                            const float e1 = lprod[2 * i + h], tk = ok ? t : 0.0f;
+                            lprod[2 * i + h] = fmaf(e1, tk, tk) + e1;
+                        } else {
+                            const float sp = fmaxf(zz, 0.0f) + log1pf(t);  // softplus(z)
+                            lsum[2 * i + h] += ok ? fmaf(yn[e], zz, -sp) : 0.0f;
+                        }
                     }
                     dst[8 * i] = make_float4(r[0], r[0], r[1], r[1]);
                 }
             }
 #pragma unroll
-            for (int c = 0; c < 8; ++c) lacc[c] = ff_add(lacc[c], lsum[c]);
+            for (int c = 0; c < 8; ++c) lacc[c] = ff_add(lacc[c], ROUND ? lsum[c] - log1pf(lprod[c]) : lsum[c]);
         };
         if (row0 + TN <= r_end) epilogue(std::true_type{});
         else epilogue(std::false_type{});
@@ -407,7 +446,7 @@ size_t f32_smem(bool packed) {
 }
 
 template <int KP>
-cudaError_t launch_f32(const LogregData& D, const float* W, int64_t M, int S, float* gpart,
+cudaError_t launch_f32(const LogregData& D, const float* W, int64_t M, int S, bool round_lp, float* gpart,
                        float2* lpart, cudaStream_t st, const int* guard) {
     const int rps = (D.n + S - 1) / S;
     const dim3 grid((unsigned)((M + TM - 1) / TM), (unsigned)S);
@@ -418,10 +457,10 @@ cudaError_t launch_f32(const LogregData& D, const float* W, int64_t M, int S, fl
         if (e != cudaSuccess) return e;
         if ((int64_t)grid.x * S > nsm) {
             const size_t smem = f32_smem<KP>(true);
-            e = cudaFuncSetAttribute(logreg_grad_f32p_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            auto fn = round_lp ? logreg_grad_f32p_kernel<KP, true> : logreg_grad_f32p_kernel<KP, false>;
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            logreg_grad_f32p_kernel<KP><<<grid, PT, smem, st>>>(W, M, D.X, D.y, D.n, (D.d + 3) / 4 * 4, rps, D.inv_v,
-                                                                gpart, lpart, guard);
+            fn<<<grid, PT, smem, st>>>(W, M, D.X, D.y, D.n, (D.d + 3) / 4 * 4, rps, D.inv_v, gpart, lpart, guard);
             return cudaGetLastError();
         }
     }
@@ -475,15 +514,15 @@ int logreg_f32_splits(const LogregData& D, int64_t M, int nsm) {
     return best;
 }
 
-cudaError_t logreg_grad_f32(const LogregData& D, const float* W, int64_t M, int S, float* gpart,
+cudaError_t logreg_grad_f32(const LogregData& D, const float* W, int64_t M, int S, bool round_lp, float* gpart,
                             float2* lpart, cudaStream_t st, const int* guard) {
     if (M <= 0) return cudaSuccess;
     if (S < 1 || S > 65535 || (M + TM - 1) / TM > 0x7fffffff) return cudaErrorInvalidValue;
     switch (D.kp) {
-    case 64: return launch_f32<64>(D, W, M, S, gpart, lpart, st, guard);
-    case 128: return launch_f32<128>(D, W, M, S, gpart, lpart, st, guard);
-    case 192: return launch_f32<192>(D, W, M, S, gpart, lpart, st, guard);
-    case 256: return launch_f32<256>(D, W, M, S, gpart, lpart, st, guard);
+    case 64: return launch_f32<64>(D, W, M, S, round_lp, gpart, lpart, st, guard);
+    case 128: return launch_f32<128>(D, W, M, S, round_lp, gpart, lpart, st, guard);
+    case 192: return launch_f32<192>(D, W, M, S, round_lp, gpart, lpart, st, guard);
+    case 256: return launch_f32<256>(D, W, M, S, round_lp, gpart, lpart, st, guard);
     }
     return cudaErrorInvalidValue;
 }

@@ -74,7 +74,9 @@ cudaError_t logreg_grad_x3(const LogregData& D, const float* W32, int64_t M, int
 // an optional guard: a device word that a launch earlier on the stream set to 0
 // when this evaluation belongs to an iteration that no longer runs (past a stop
 // or a switch); the kernel then returns at once.
-cudaError_t logreg_grad_f32(const LogregData& D, const float* W, int64_t M, int S, float* gpart,
+// round_lp: the caller rounds log p to binary32 (a target call): its sum need not be the
+// sampler's bit for bit.
+cudaError_t logreg_grad_f32(const LogregData& D, const float* W, int64_t M, int S, bool round_lp, float* gpart,
                             float2* lpart, cudaStream_t st, const int* guard = nullptr);
 // The data split S of logreg_grad_f32 for M points on nsm SMs: the number of row
 // ranges (1 .. 16) that minimises waves of blocks x rows per block, so that the

@@ -487,7 +487,7 @@ laps_status launch_grad(laps_ctx* c, int form, cudaStream_t st, const int* guard
         e = logreg_grad_x3(c->tg->lr, c->W, c->M, c->nsplit_x3, c->rps_x3, c->gpart, c->lpart, c->status,
                            c->cfg.barrier_timeout_ns, st, guard);
     else
-        e = logreg_grad_f32(c->tg->lr, c->W, c->M, c->nsplit, c->gpart, c->lpart, st, guard);
+        e = logreg_grad_f32(c->tg->lr, c->W, c->M, c->nsplit, false, c->gpart, c->lpart, st, guard);
     return e == cudaSuccess ? LAPS_OK
                             : cuda_fail(e, form == GF_BF16 ? "logreg gradient (tensor cores)"
                                            : form == GF_X3 ? "logreg gradient (tensor cores, three-term split)"
@@ -771,7 +771,7 @@ laps_status streamed_target_grad(const laps_target* tg, const float* W, int64_t 
         cudaError_t e = gauss_dense_grad(tg->prec_dense, tg->d_pad, tg->d, W, M, gpart, lpart, st);
         return e == cudaSuccess ? LAPS_OK : cuda_fail(e, "dense Gaussian gradient");
     }
-    cudaError_t e = logreg_grad_f32(tg->lr, W, M, S, gpart, lpart, st);
+    cudaError_t e = logreg_grad_f32(tg->lr, W, M, S, true, gpart, lpart, st);
     return e == cudaSuccess ? LAPS_OK : cuda_fail(e, "logreg gradient");
 }
 

@@ -11,7 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,d,M", [(1, 2, 1), (63, 3, 63), (64, 4, 64), (65, 5, 65), (128, 63, 2), (129, 64, 129),
-                                   (200, 65, 64), (999, 124, 130), (1000, 125, 7), (5000, 128, 200)])
+                                   (200, 65, 64), (999, 124, 130), (1000, 125, 7), (5000, 128, 200),
+                                   # grids of more blocks than SMs, where the packed kernel runs
+                                   (1000, 125, 641), (65, 64, 4990), (130, 3, 3300), (2, 2, 9800), (999, 128, 700),
+                                   (64, 65, 9729), (190, 63, 3265)])
 def test_gradient_at_tile_edges(ora, n, d, M):
     from paper_2601_16696_gb300 import laps
     pr = W.logreg(n_data=max(n, 2), n_feat=d - 1, M=M, data_seed=n + d)
