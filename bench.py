@@ -396,7 +396,7 @@ def _forms(flush, stream, mhz, seed0):
     flops = 4.0 * pr.M * n * pr.d  # Z = W X^T and G = R X per gradient of the ensemble
     lr = {"workload": "logreg_d%d_n%d_M%d_%dsteps" % (pr.d, n, pr.M, pr.n_steps),
           "b2": "b2_max", "truth": truth, "switch": "paper rule (max delta < 0.01)"}
-    kernels = {0: "logreg_grad_f32_kernel<128>", 1: "logreg_grad_mma_kernel<128>",
+    kernels = {0: "logreg_grad_f32p_kernel<128>", 1: "logreg_grad_mma_kernel<128>",
                2: "logreg_grad_x3_kernel<128>"}
     for name, prec in (("mixed", 1), ("fp32", 0), ("bf16x3", 2)):
         for _ in range(3):
@@ -483,7 +483,7 @@ def _forms(flush, stream, mhz, seed0):
                      "kernel": "gauss_dense_grad_kernel<4,2> (the streamed path's gradient)",
                      "timed": "laps_target_logp_grad (points packed, contraction, partials "
                               "unpacked), %.3f ms per call; 2 M d^2 algorithmic FLOP, the "
-                              "compensated accumulation's extra operations not counted" % gms,
+                              "biased accumulation's extra operations not counted" % gms,
                      "peak_basis": "%d SMs x 128 FP32 FMA lanes x 2 x %.0f MHz" % (nsm, mhz)}}
     # ---- the full-rank bias proxy: unadjusted iterations on the headline ensemble
     pr = workloads.banana()

@@ -180,8 +180,8 @@ __device__ __forceinline__ void g_o(const KParams& P, const PhiloxKeys& K, Grp& 
 }
 
 // The elementwise operations run on pairs of coordinates (add/mul/fma.rn.f32x2: one issue
-// slot for two; the step loop issues in 53-57% of its slots with one block an SM); the sums
-// over a lane's coordinates are added one by one in order, so that every result keeps its
+// slot for two; with one block an SM the step loop issues in 51% of its slots, 53-57% before
+// with 8-13% more instructions); the sums over a lane's coordinates are added one by one in order, so that every result keeps its
 // bits.  Measured: a d = 10^4 problem (4096 chains) with 24 small ones, 8 unadjusted
 // iterations 6273 -> 6124 us; small problems alone, adjusted proposals 1318 -> 1279 us.
 //

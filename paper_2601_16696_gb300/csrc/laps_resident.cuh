@@ -85,7 +85,7 @@ __device__ __forceinline__ void dense_px_comp(const float* sP, float* sx, int d,
 // lanes stage their coordinates of x in the slot's row; each lane then forms its
 // coordinates of P x over the d columns, reading row j of the symmetric P for column j
 // (float4 reads, consecutive across the group's lanes).  Measured at d = 100, M = 4096
-// (register-resident): 45 us per unadjusted step with the compensated form, 31 us now,
+// (register-resident): 42 us per unadjusted step with the compensated form, 27 us now,
 // of which about 19 us are these products.
 template <int LPC, int CPL>
 __device__ __forceinline__ void dense_px(const KParams& P, int gl, float* dsm, const float (&x)[CPL],
