@@ -483,7 +483,7 @@ def _forms(flush, stream, mhz, seed0):
                      "kernel": "gauss_dense_grad_kernel<4,2> (the streamed path's gradient)",
                      "timed": "laps_target_logp_grad (points packed, contraction, partials "
                               "unpacked), %.3f ms per call; 2 M d^2 algorithmic FLOP, the "
-                              "biased accumulation's extra operations not counted" % gms,
+                              "compensated accumulation's extra operations not counted" % gms,
                      "peak_basis": "%d SMs x 128 FP32 FMA lanes x 2 x %.0f MHz" % (nsm, mhz)}}
     # ---- the full-rank bias proxy: unadjusted iterations on the headline ensemble
     pr = workloads.banana()

@@ -390,13 +390,11 @@ laps_status laps_target_create(const laps_target_desc* desc, laps_target** out) 
         // padded to whole 32-column tiles of the contraction; padding rows and columns are zero
         t->d_pad = (int)((d + 31) / 32 * 32);
         const size_t pb = (size_t)t->d_pad * t->d_pad * sizeof(float);
-        cudaError_t e = cudaMalloc(&t->prec_dense, pb + t->d_pad * sizeof(float));
+        cudaError_t e = cudaMalloc(&t->prec_dense, pb);
         if (e == cudaSuccess) e = cudaMemset(t->prec_dense, 0, pb);
         if (e == cudaSuccess)
             e = cudaMemcpy2D(t->prec_dense, t->d_pad * sizeof(float), desc->prec, d * sizeof(float),
                              d * sizeof(float), d, cudaMemcpyDeviceToDevice);
-        if (e == cudaSuccess) e = dense_row_norms(t->prec_dense, t->d_pad, nullptr);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
         if (e != cudaSuccess) {
             laps_target_destroy(t);
             return cuda_fail(e, "GAUSS_DENSE precision copy");

@@ -6,19 +6,22 @@
 // A block owns a few chains per warp (CW x warps, launch_q): their points stay in
 // shared memory as pairs (x_k, x_k), P streams through shared memory kRows rows at a
 // time (two buffers, cp.async), and lane l of the chain's warp accumulates the column
-// pairs 2 l + 64 p in packed arithmetic.
+// pairs 2 l + 64 p in packed arithmetic (an odd multiple of 32 columns leaves one column
+// a lane, in scalar arithmetic: a pair would idle half the warp).
 //
 // The target is ill-conditioned (condition number ~1e5 in the paper's
 // experiment), so -P x cancels: a binary32 dot product loses ~1e-4 of max|g|.
-// The sums run in the biased form of laps_resident.cuh (dense_bias_add: four
-// operations per product); a chain whose result is too small against its bias for
-// that form's accuracy (dense_bias_ok) is recomputed in the compensated form, in a
-// second pass of its block.  log p sums x_o (P x)_o compensated, one warp butterfly
-// per chain.
+// Each product therefore enters exactly into a float-float accumulator, two columns
+// at a time (dense_add in laps_resident.cuh): the result is as accurate as a dot
+// product in twice the working precision, rounded once.  log p sums x_o (P x)_o the
+// same way, one warp butterfly per chain.
 //
-// Bound by the FMA pipe (4 M d d_pad operations) and the operand loads: M = 1500,
-// d = 300 takes 38 us, 91 us before (scalar compensated sums of ten operations a
-// product, 188 blocks on 152 SMs).
+// What bounds it: ten FMA-pipe operations a product, and next to them the latency of the
+// operand loads and of the sums' chains with one block of ten to sixteen warps an SM (M = 1500,
+// d = 300: FMA pipe 58% busy, issue slots 40%).  Measured, us a launch, against scalar sums with
+// a fixed sixteen chains a block (188 blocks on 152 SMs there): M = 1500, d = 300 88 -> 62;
+// M = 4096, d = 200 79 -> 73; M = 4096, d = 100 24.5 -> 24.1.  The figures do not depend on the
+// condition number.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -31,9 +34,9 @@ namespace {
 constexpr int kRows = 16;       // rows of P per chunk (d_pad is a multiple of 32)
 constexpr int kMaxWarps = 16;
 
-// W [M][dp] points (zero padded), P [dp][dp] symmetric (zero padded) and its row norms
-// [dp], dp = 32 Q.  G [M][dp] receives -P x (zeros in the padding), LP [M] log p as
-// float-float.  nw: warps that hold chains (the block's other warps only stage).
+// W [M][dp] points (zero padded), P [dp][dp] symmetric (zero padded), dp = 32 Q.
+// G [M][dp] receives -P x (zeros in the padding), LP [M] log p as float-float.
+// nw: warps that hold chains (the block's other warps only stage).
 template <int Q, int CW>
 __global__ void __launch_bounds__(32 * kMaxWarps) gauss_dense_grad_kernel(const float* __restrict__ P, int d,
                                                                      const float* __restrict__ W, int64_t M, int nw,
@@ -41,7 +44,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) gauss_dense_grad_kernel(const 
                                                                      float2* __restrict__ LP,
                                                                      const int* __restrict__ guard) {
     if (guard != nullptr && *guard == 0) return;  // the iteration no longer runs
-    constexpr int dp = 32 * Q, NP = (Q + 1) / 2;
+    constexpr int dp = 32 * Q, NP = Q / 2;  // pairs a lane; odd Q: one more column
     extern __shared__ __align__(16) float sm[];
     const int nch = nw * CW;
     float* Xs = sm;                    // [nch][2 dp] pairs
@@ -68,39 +71,80 @@ __global__ void __launch_bounds__(32 * kMaxWarps) gauss_dense_grad_kernel(const 
     __syncthreads();  // the points are staged
     const int ch0 = CW * warp;           // this warp's first chain (warp < nw)
     const bool work = warp < nw;
-    const bool tail = Q % 2 == 0 || lane < 16;  // odd Q: the last pair exists for 16 lanes
-    // one pass over P's rows: row(kk, x pairs of two rows per chain offset, chunk)
-    auto stream = [&](auto&& body) {
-        for (int k0 = 0, b = 0; k0 < d; k0 += kRows, b ^= 1) {
-            if (k0 + kRows < d) {
-                stage(k0 + kRows, b ^ 1);
-                asm volatile("cp.async.wait_group 1;" ::: "memory");
-            } else {
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-            }
-            __syncthreads();
-            // rows past d of P are zero: they would add exact zeros, so stop at d (rounded up to 2)
-            const int kn = d - k0 < kRows ? d - k0 : kRows;
-            if (work) body(k0, kn, Ps + b * kRows * dp + 2 * lane);
-            __syncthreads();  // the buffer may be overwritten
+    f32x2 hi[CW][NP + 1], lo[CW][NP + 1];
+    float hi1[CW], lo1[CW];
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+        hi1[c] = lo1[c] = 0.0f;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) hi[c][p] = lo[c][p] = 0;
+    }
+    const f32x2 m1 = pack2(-1.0f, -1.0f);
+    for (int k0 = 0, b = 0; k0 < d; k0 += kRows, b ^= 1) {
+        if (k0 + kRows < d) {
+            stage(k0 + kRows, b ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
-    };
-    // -P x of one chain and its log p
-    auto finish = [&](int ch, const float (&r)[2 * NP]) {
+        __syncthreads();
+        // rows past d of P are zero: they would add exact zeros, so stop at d (rounded up to 2)
+        const int kn = work ? min(kRows, d - k0) : 0;
+        const float *Pc = Ps + b * kRows * dp + 2 * lane, *P1 = Ps + b * kRows * dp + 64 * NP + lane;
+#pragma unroll 2
+        for (int kk = 0; kk < kn; kk += 2) {
+            ulonglong2 xx[CW], nx[CW];
+#pragma unroll
+            for (int c = 0; c < CW; ++c) {
+                xx[c] = *reinterpret_cast<const ulonglong2*>(Xs + (ch0 + c) * 2 * dp + 2 * (k0 + kk));
+                nx[c] = make_ulonglong2(mul2(xx[c].x, m1), mul2(xx[c].y, m1));
+            }
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const f32x2 p0 = *reinterpret_cast<const f32x2*>(Pc + kk * dp + 64 * p);
+                const f32x2 p1 = *reinterpret_cast<const f32x2*>(Pc + (kk + 1) * dp + 64 * p);
+#pragma unroll
+                for (int c = 0; c < CW; ++c) {
+                    dense_add(xx[c].x, nx[c].x, p0, m1, hi[c][p], lo[c][p]);
+                    dense_add(xx[c].y, nx[c].y, p1, m1, hi[c][p], lo[c][p]);
+                }
+            }
+            if constexpr (Q % 2 == 1) {
+                const float p0 = P1[kk * dp], p1 = P1[(kk + 1) * dp];
+#pragma unroll
+                for (int c = 0; c < CW; ++c) {
+                    dense_add(unpack2(xx[c].x).x, p0, hi1[c], lo1[c]);
+                    dense_add(unpack2(xx[c].y).x, p1, hi1[c], lo1[c]);
+                }
+            }
+        }
+        __syncthreads();  // the buffer may be overwritten
+    }
+    if (!work) return;
+    // -P x of each chain and its log p
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+        const int ch = ch0 + c;
+        const float* xs = Xs + ch * 2 * dp;
         ff l = ff_make(0.0f);
+        auto add_lp = [&](int o, float r) {
+            const float pr = xs[2 * o] * r;
+            l = ff_add(l, ff{pr, fmaf(xs[2 * o], r, -pr)});
+        };
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            if (p == NP - 1 && !tail) continue;
             const int o = 2 * lane + 64 * p;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float xo = Xs[ch * 2 * dp + 2 * (o + e)], rv = r[2 * p + e];
-                const float pr = xo * rv;
-                l = ff_add(l, ff{pr, fmaf(xo, rv, -pr)});
-            }
+            const float2 r = unpack2(add2(hi[c][p], lo[c][p]));
+            add_lp(o, r.x);
+            add_lp(o + 1, r.y);
             if (ch < nc)
-                *reinterpret_cast<float2*>(G + (m0 + ch) * dp + o) =
-                    make_float2(o < d ? -r[2 * p] : 0.0f, o + 1 < d ? -r[2 * p + 1] : 0.0f);
+                *reinterpret_cast<float2*>(G + (m0 + ch) * dp + o) = make_float2(o < d ? -r.x : 0.0f, o + 1 < d ? -r.y : 0.0f);
+        }
+        if constexpr (Q % 2 == 1) {
+            const int o = 64 * NP + lane;
+            const float r = hi1[c] + lo1[c];
+            add_lp(o, r);
+            if (ch < nc) G[(m0 + ch) * dp + o] = o < d ? -r : 0.0f;
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
@@ -108,108 +152,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) gauss_dense_grad_kernel(const 
             l = ff_add(l, w);
         }
         if (lane == 0 && ch < nc) LP[m0 + ch] = make_float2(-0.5f * l.hi, -0.5f * l.lo);
-    };
-
-    f32x2 S[CW][NP], lo[CW][NP];
-    float nx[CW];
-    const float2* sn = reinterpret_cast<const float2*>(P + (size_t)dp * dp) + lane;
-#pragma unroll
-    for (int c = 0; c < CW; ++c) {
-        float n2 = 0.0f;
-        if (work)
-            for (int o = lane; o < d; o += 32) n2 = fmaf(Xs[(ch0 + c) * 2 * dp + 2 * o], Xs[(ch0 + c) * 2 * dp + 2 * o], n2);
-        nx[c] = sqrtf(group_sum<32>(n2));
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            const float2 np = p < NP - 1 || tail ? sn[32 * p] : make_float2(0.0f, 0.0f);
-            S[c][p] = pack2(dense_sigma(nx[c], np.x), dense_sigma(nx[c], np.y));
-            lo[c][p] = 0;
-        }
     }
-    const f32x2 m1 = pack2(-1.0f, -1.0f);
-    stream([&](int k0, int kn, const float* Pc) {
-#pragma unroll 2
-        for (int kk = 0; kk < kn; kk += 2) {
-            ulonglong2 xx[CW];
-#pragma unroll
-            for (int c = 0; c < CW; ++c) xx[c] = *reinterpret_cast<const ulonglong2*>(Xs + (ch0 + c) * 2 * dp + 2 * (k0 + kk));
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                f32x2 p0 = 0, p1 = 0;
-                if (p < NP - 1 || tail) {
-                    p0 = *reinterpret_cast<const f32x2*>(Pc + kk * dp + 64 * p);
-                    p1 = *reinterpret_cast<const f32x2*>(Pc + (kk + 1) * dp + 64 * p);
-                }
-#pragma unroll
-                for (int c = 0; c < CW; ++c) {
-                    dense_bias_add(xx[c].x, p0, m1, S[c][p], lo[c][p]);
-                    dense_bias_add(xx[c].y, p1, m1, S[c][p], lo[c][p]);
-                }
-            }
-        }
-    });
-    unsigned again = 0u;  // bit c: chain c of this warp needs the compensated form
-    if (work) {
-#pragma unroll
-        for (int c = 0; c < CW; ++c) {
-            float r[2 * NP], rmax = 0.0f, smax = 0.0f;
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const float2 np = p < NP - 1 || tail ? sn[32 * p] : make_float2(0.0f, 0.0f);
-                const float s0 = dense_sigma(nx[c], np.x), s1 = dense_sigma(nx[c], np.y);
-                const float2 Sv = unpack2(S[c][p]), lv = unpack2(lo[c][p]);
-                r[2 * p] = (Sv.x - s0) + lv.x;
-                r[2 * p + 1] = (Sv.y - s1) + lv.y;
-                rmax = fmaxf(rmax, fmaxf(fabsf(r[2 * p]), fabsf(r[2 * p + 1])));
-                smax = fmaxf(smax, fmaxf(s0, s1));
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, off));
-                smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, off));
-            }
-            if ((!dense_bias_ok(rmax, smax) || !(nx[c] < 3e38f)) && ch0 + c < nc) {
-                bool nz = false;  // x = 0 needs no repeat: its r is exactly 0
-                for (int o = lane; o < d; o += 32) nz = nz || Xs[(ch0 + c) * 2 * dp + 2 * o] != 0.0f;
-                if (__any_sync(0xffffffffu, nz)) again |= 1u << c;
-            }
-            finish(ch0 + c, r);
-        }
-    }
-    if (!__syncthreads_or((int)again)) return;
-    for (int c = 0; c < CW; ++c) {  // rare: another pass of the block per chain slot
-        stage(0, 0);
-        float hi[2 * NP], lw[2 * NP];
-#pragma unroll
-        for (int q = 0; q < 2 * NP; ++q) hi[q] = lw[q] = 0.0f;
-        stream([&](int k0, int kn, const float* Pc) {
-            for (int kk = 0; kk < kn; ++kk) {
-                const float x = Xs[(ch0 + c) * 2 * dp + 2 * (k0 + kk)];
-#pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    if (p == NP - 1 && !tail) continue;
-                    const float2 pv = *reinterpret_cast<const float2*>(Pc + kk * dp + 64 * p);
-                    dense_comp_add(x, pv.x, hi[2 * p], lw[2 * p]);
-                    dense_comp_add(x, pv.y, hi[2 * p + 1], lw[2 * p + 1]);
-                }
-            }
-        });
-        if ((again >> c) & 1u) {
-#pragma unroll
-            for (int q = 0; q < 2 * NP; ++q) hi[q] += lw[q];
-            finish(ch0 + c, hi);
-        }
-    }
-}
-
-// |P_i| of every row (and, P being symmetric, column), one warp per row
-__global__ void dense_row_norms_kernel(float* __restrict__ P, int dp) {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (i >= dp) return;
-    float a = 0.0f;
-    for (int j = lane; j < dp; j += 32) a = fmaf(P[(size_t)i * dp + j], P[(size_t)i * dp + j], a);
-    a = group_sum<32>(a);
-    if (lane == 0) P[(size_t)dp * dp + i] = sqrtf(a);
 }
 
 // Chains per block: an SM holds one block, so the ensemble is split evenly over the
@@ -243,11 +186,6 @@ cudaError_t launch_q(const float* P, int d, const float* W, int64_t M, float* G,
     return launch_cw<Q, 2>(P, d, W, M, per_sm, G, LP, st, guard);
 }
 }  // namespace
-
-cudaError_t dense_row_norms(float* P, int d_pad, cudaStream_t st) {
-    dense_row_norms_kernel<<<(d_pad * 32 + 255) / 256, 256, 0, st>>>(P, d_pad);
-    return cudaGetLastError();
-}
 
 cudaError_t gauss_dense_grad(const float* P, int d_pad, int d, const float* W, int64_t M, float* G,
                              float2* LP, cudaStream_t st, const int* guard) {

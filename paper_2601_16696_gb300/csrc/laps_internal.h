@@ -14,7 +14,7 @@ struct laps_target {
     int kind = 0, d = 0, d_pad = 0;
     float* prec_pad = nullptr;  // GAUSS_DIAG precisions, zero padded to d_pad (owned)
     laps::LogregData lr{};      // LOGREG: padded copies of X and y (owned)
-    float* prec_dense = nullptr; // GAUSS_DENSE: P [d_pad][d_pad], zero padded, d_pad = 32 k, then |P_i| [d_pad] (owned)
+    float* prec_dense = nullptr; // GAUSS_DENSE: P [d_pad][d_pad], zero padded, d_pad = 32 k (owned)
     int* status = nullptr;      // LOGREG: latched status of the tensor-core target call (owned)
 };
 
@@ -138,9 +138,7 @@ constexpr int kDenseMaxDim = 512;
 // forms of the logistic-regression contraction: FP32 on the CUDA cores, BF16
 // tensor cores, tensor cores at FP32 accuracy (three-term BF16 split)
 enum GradForm : int { GF_F32 = 0, GF_BF16 = 1, GF_X3 = 2 };
-// (guard: as for the logistic-regression gradients, laps_logreg.cuh).  P is followed by
-// the norms of its rows, which dense_row_norms writes.
-cudaError_t dense_row_norms(float* P, int d_pad, cudaStream_t st);
+// (guard: as for the logistic-regression gradients, laps_logreg.cuh)
 cudaError_t gauss_dense_grad(const float* P, int d_pad, int d, const float* W, int64_t M, float* G,
                              float2* LP, cudaStream_t st, const int* guard = nullptr);
 inline bool streamed_kind(int kind) { return kind == TGT_LOGREG || kind == TGT_GAUSS_DENSE || kind == TGT_USER; }

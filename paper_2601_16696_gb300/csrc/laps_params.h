@@ -132,10 +132,10 @@ __host__ __device__ inline int fr_jsplit(int d_pad, int slots, int K, int thread
     return js > 1 ? js : 1;
 }
 // shared memory of the dense-precision Gaussian on the resident kernel (bytes,
-// after the reduction's slice rows): 16 bytes of alignment, P [d_pad][d_pad], the
-// norms of its rows [d_pad] and one row of pairs (x_j, x_j) [2 d_pad] per chain slot
+// after the reduction's slice rows): 16 bytes of alignment, P [d_pad][d_pad] and one
+// row of pairs (x_j, x_j) [2 d_pad] per chain slot
 __host__ __device__ inline size_t dense_smem(int d_pad, int slots) {
-    return 16 + 4 * ((size_t)d_pad * d_pad + d_pad + (size_t)slots * 2 * d_pad);
+    return 16 + 4 * ((size_t)d_pad * d_pad + (size_t)slots * 2 * d_pad);
 }
 // the largest padded dimension the resident kernel serves it for (P in shared memory)
 constexpr int kDenseResidentMax = 128;

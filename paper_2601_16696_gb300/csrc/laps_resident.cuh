@@ -23,79 +23,49 @@ struct Coefs {  // integrator tables (Table "integrators"), copied to shared mem
 // ---------------------------------------------------------------- target
 // Dense-precision Gaussian (Sec. 6, the rotated ill-conditioned Gaussian): a dot
 // product sum_j x_j P_ji that keeps twice binary32's precision, since at condition
-// numbers near 1e5 a binary32 sum loses ~1e-4 of the gradient to cancellation.
-//
-// Biased form (DenseBias): the accumulator S starts at sigma = 1.5 2^k with 2^(k-1)
-// above a bound of every partial sum (Cauchy-Schwarz, |x| |P_i|), so S stays in
-// (2^k, 2^(k+1)) and |S| exceeds every product.  Then s = fma(x, p, S) has the
-// rounding error e = x p - (s - S) with s - S exact (Dekker's fast two-sum applied to
-// the unrounded product), and e = fma(x, p, S - s): four operations per product where
-// the compensated product and sum (Ogita, Rump and Oishi, 2005) take ten.  What is
-// dropped is the rounding of e and of their sum, about 2^-42 sigma in all, so the
-// result is as accurate as the compensated one while max_i |r_i| >= 2^-15 sigma
-// (dense_bias_ok); past that, where the cancellation is heavier than condition numbers
-// near 1e9 give, and where sigma overflows or underflows, the caller recomputes the
-// compensated form.  Measured against 64 bits for seeds, sizes and both starts: equal
-// to it in every digit printed (2.5e-8 of |r|) up to condition 2.5e6.
-__device__ __forceinline__ float dense_sigma(float nx, float np) {
-    const uint32_t E = __float_as_uint(1.0001f * nx * np) >> 23;  // bound < 2^(E - 126)
-    return __uint_as_float(((E + 2u) << 23) | 0x400000u);
-}
-__device__ __forceinline__ bool dense_bias_ok(float rmax, float smax) {
-    return rmax * 32768.0f >= smax && smax >= 1e-25f;  // false for NaN
-}
-__device__ __forceinline__ void dense_bias_add(f32x2 x, f32x2 p, f32x2 m1, f32x2& S, f32x2& lo) {
-    const f32x2 s = fma2(x, p, S);
-    lo = add2(lo, fma2(x, p, fma2(s, m1, S)));
-    S = s;
-}
-// the compensated form of the same step: x p = pv + er exactly, (hi, sl) = TwoSum(hi, pv)
-__device__ __forceinline__ void dense_comp_add(float x, float p, float& hi, float& lo) {
-    const float pv = x * p;
-    const float er = fmaf(x, p, -pv);
-    float sh, sl;
-    two_sum(hi, pv, sh, sl);
-    hi = sh;
-    lo += sl + er;
+// numbers near 1e5 a binary32 sum loses ~1e-4 of the gradient to cancellation.  Every
+// product enters a float-float accumulator exactly, the compensated dot product of
+// Ogita, Rump and Oishi ("Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005):
+// x p = pr + er, (s, e) = TwoSum(hi, pr), lo += e + er, ten operations a product, here for
+// two columns at once (packed operations round each half as scalar ones; v - w is
+// fma(w, -1, v), pr enters as npr = (-x) p = -pr): bit for bit the scalar sums.  Not taken: four
+// operations a product with the errors rounded against a bound of |x||P_i| in place of the
+// running sum, 0.6 to 0.8 of the time below condition numbers of 1e7 and more than the scalar
+// sums' beyond: a component that is small against its chain's largest lost up to three digits,
+// and a row whose bound leaves binary32's range the compensation.
+__device__ __forceinline__ void dense_add(f32x2 x, f32x2 nx, f32x2 p, f32x2 m1, f32x2& hi, f32x2& lo) {
+    const f32x2 npr = mul2(nx, p);
+    const f32x2 er = fma2(x, p, npr);
+    const f32x2 s = fma2(npr, m1, hi);
+    const f32x2 bp = fma2(hi, m1, s);
+    const f32x2 e = fma2(add2(npr, bp), m1, fma2(fma2(bp, m1, s), m1, hi));
+    hi = s;
+    lo = add2(lo, add2(e, er));
 }
 
-// P x in the compensated form for the chain whose pairs (x_j, x_j) are at sx; the result
-// replaces the second of each pair (one coordinate block at a time: rare, few registers)
-template <int LPC, int CPL>
-__device__ __forceinline__ void dense_px_comp(const float* sP, float* sx, int d, int dp, int nblk, int gl) {
-#pragma unroll 1
-    for (int j = gl; j < nblk; j += LPC) {
-        float hi[4] = {0.0f, 0.0f, 0.0f, 0.0f}, lo[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 1
-        for (int jj = 0; jj < d; ++jj) {
-            const float xj = sx[2 * jj];
-            const float4 p4 = *reinterpret_cast<const float4*>(sP + (size_t)jj * dp + 4 * j);
-            dense_comp_add(xj, p4.x, hi[0], lo[0]);
-            dense_comp_add(xj, p4.y, hi[1], lo[1]);
-            dense_comp_add(xj, p4.z, hi[2], lo[2]);
-            dense_comp_add(xj, p4.w, hi[3], lo[3]);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) sx[8 * j + 2 * c + 1] = hi[c] + lo[c];
-    }
+// the same for one column
+__device__ __forceinline__ void dense_add(float x, float p, float& hi, float& lo) {
+    const float pr = x * p, er = fmaf(x, p, -pr);
+    float s, e;
+    two_sum(hi, pr, s, e);
+    hi = s;
+    lo += e + er;
 }
 
-// r = P x for the group's chain.  dsm holds P [d_pad][d_pad], the norms of its rows
-// [d_pad], then one row of pairs (x_j, x_j) [2 d_pad] per chain slot of the block.  The
-// lanes stage their coordinates of x in the slot's row; each lane then forms its
-// coordinates of P x over the d columns, reading row j of the symmetric P for column j
-// (float4 reads, consecutive across the group's lanes).  Measured at d = 100, M = 4096
-// (register-resident): 42 us per unadjusted step with the compensated form, 27 us now,
-// of which about 19 us are these products.
+// r = P x for the group's chain.  dsm holds P [d_pad][d_pad], then one row of pairs
+// (x_j, x_j) [2 d_pad] per chain slot of the block.  The lanes stage their coordinates of
+// x in the slot's row; each lane then forms its coordinates of P x over the d columns,
+// reading row j of the symmetric P for column j (16-byte reads, consecutive across the
+// group's lanes).  Measured at d = 100, start and 16 unadjusted steps, scalar sums against these
+// pairs: M = 4096 744 -> 640 us, M = 1024 749 -> 493 us; start and one adjusted proposal of 15
+// steps, M = 4096 1180 -> 924 us; the same at condition numbers 1e5 to 1e8.
 template <int LPC, int CPL>
 __device__ __forceinline__ void dense_px(const KParams& P, int gl, float* dsm, const float (&x)[CPL],
                                          float (&r)[CPL]) {
     constexpr int NB = CPL / 4;
     const int dp = P.d_pad;
     const float* sP = dsm;
-    const float* sn = dsm + (size_t)dp * dp;
-    float* sx = dsm + (size_t)dp * dp + dp + (size_t)(threadIdx.x / LPC) * 2 * dp;
-    float n2 = 0.0f;
+    float* sx = dsm + (size_t)dp * dp + (size_t)(threadIdx.x / LPC) * 2 * dp;
 #pragma unroll
     for (int k = 0; k < NB; ++k) {
         const int j = gl + LPC * k;
@@ -104,79 +74,36 @@ __device__ __forceinline__ void dense_px(const KParams& P, int gl, float* dsm, c
             dst[0] = make_float4(x[4 * k], x[4 * k], x[4 * k + 1], x[4 * k + 1]);
             dst[1] = make_float4(x[4 * k + 2], x[4 * k + 2], x[4 * k + 3], x[4 * k + 3]);
         }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) n2 = fmaf(x[4 * k + c], x[4 * k + c], n2);
     }
-    const float nx = sqrtf(group_sum<LPC>(n2));
     __syncwarp();
-    f32x2 S[2 * NB], lo[2 * NB];
+    f32x2 hi[2 * NB], lo[2 * NB];
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-        const int j = gl + LPC * k;
-        float4 np = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (j < P.nblk) np = *reinterpret_cast<const float4*>(sn + 4 * j);
-        S[2 * k] = pack2(dense_sigma(nx, np.x), dense_sigma(nx, np.y));
-        S[2 * k + 1] = pack2(dense_sigma(nx, np.z), dense_sigma(nx, np.w));
-        lo[2 * k] = lo[2 * k + 1] = 0;
-    }
+    for (int k = 0; k < 2 * NB; ++k) hi[k] = lo[k] = 0;
     const f32x2 m1 = pack2(-1.0f, -1.0f);
     const int nb_live = P.nblk - gl;  // block k of this lane exists while LPC k < nb_live
 #pragma unroll 1
-    for (int jj = 0; jj < P.d; jj += 2) {  // rows past d are zero
+    for (int jj = 0; jj < P.d; jj += 2) {  // rows past d are zero: they add exact zeros
         const ulonglong2 xx = *reinterpret_cast<const ulonglong2*>(sx + 2 * jj);
+        const f32x2 n0 = mul2(xx.x, m1), n1 = mul2(xx.y, m1);
 #pragma unroll
         for (int k = 0; k < NB; ++k) {
             if (LPC * k >= nb_live) continue;
             const float* row = sP + (size_t)jj * dp + 4 * (gl + LPC * k);
             const ulonglong2 p0 = *reinterpret_cast<const ulonglong2*>(row);
             const ulonglong2 p1 = *reinterpret_cast<const ulonglong2*>(row + dp);
-            dense_bias_add(xx.x, p0.x, m1, S[2 * k], lo[2 * k]);
-            dense_bias_add(xx.x, p0.y, m1, S[2 * k + 1], lo[2 * k + 1]);
-            dense_bias_add(xx.y, p1.x, m1, S[2 * k], lo[2 * k]);
-            dense_bias_add(xx.y, p1.y, m1, S[2 * k + 1], lo[2 * k + 1]);
+            dense_add(xx.x, n0, p0.x, m1, hi[2 * k], lo[2 * k]);
+            dense_add(xx.x, n0, p0.y, m1, hi[2 * k + 1], lo[2 * k + 1]);
+            dense_add(xx.y, n1, p1.x, m1, hi[2 * k], lo[2 * k]);
+            dense_add(xx.y, n1, p1.y, m1, hi[2 * k + 1], lo[2 * k + 1]);
         }
-    }
-    float rmax = 0.0f, smax = 0.0f;
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {
-        const int j = gl + LPC * k;
-        float4 np = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (j < P.nblk) np = *reinterpret_cast<const float4*>(sn + 4 * j);
-        const float nq[4] = {np.x, np.y, np.z, np.w};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float2 Sv = unpack2(S[2 * k + h]), lv = unpack2(lo[2 * k + h]);
-            const float s0 = dense_sigma(nx, nq[2 * h]), s1 = dense_sigma(nx, nq[2 * h + 1]);
-            const float r0 = (Sv.x - s0) + lv.x, r1 = (Sv.y - s1) + lv.y;
-            r[4 * k + 2 * h] = r0;
-            r[4 * k + 2 * h + 1] = r1;
-            rmax = fmaxf(rmax, fmaxf(fabsf(r0), fabsf(r1)));
-            smax = fmaxf(smax, fmaxf(s0, s1));
-        }
-    }
-#pragma unroll
-    for (int o = LPC / 2; o > 0; o >>= 1) {
-        rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-        smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-    }
-    bool again = !dense_bias_ok(rmax, smax) || !(nx < 3e38f);
-    if (__any_sync(0xffffffffu, again)) {
-        bool nz = false;  // x = 0 (an idle group too) needs no repeat: its r is exactly 0
-        for (int i = gl; i < P.d; i += LPC) nz = nz || sx[2 * i] != 0.0f;
-        const unsigned lanes = ((LPC == 32) ? 0xffffffffu : ((1u << LPC) - 1u)) << ((threadIdx.x & 31) & ~(LPC - 1));
-        const unsigned live = __ballot_sync(0xffffffffu, nz) & lanes;  // every lane of the warp votes
-        again = again && live != 0u;
-    }
-    if (__any_sync(0xffffffffu, again)) {  // rare: the whole warp repeats, only the flagged chains take the result
-        dense_px_comp<LPC, CPL>(sP, sx, P.d, dp, P.nblk, gl);
-        if (again)
-#pragma unroll
-            for (int k = 0; k < NB; ++k)
-                if (LPC * k < nb_live)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) r[4 * k + c] = sx[8 * (gl + LPC * k) + 2 * c + 1];
     }
     __syncwarp();  // the slot's row is rewritten by the next evaluation
+#pragma unroll
+    for (int k = 0; k < 2 * NB; ++k) {
+        const float2 v = unpack2(add2(hi[k], lo[k]));
+        r[2 * k] = v.x;
+        r[2 * k + 1] = v.y;
+    }
 }
 
 // log p at x = sigma o y and the gradient in y (sigma o grad_x).  Returns the

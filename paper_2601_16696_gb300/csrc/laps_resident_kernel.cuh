@@ -260,13 +260,13 @@ __global__ void __launch_bounds__(kMaxThreads) laps_resident_kernel(const KParam
     float* f_my = f_s + (size_t)slots * K4;                  // [dp] shift ybar'
     float* f_mg = f_my + dp;                                 // [dp] shift gbar'
     uint32_t* f_z = reinterpret_cast<uint32_t*>(f_mg + dp);  // [nzw][K4] Rademacher words
-    // dense-precision Gaussian only: P [dp][dp] and the norms of its rows [dp], then one
-    // row of pairs (x_j, x_j) per chain slot, after the reduction's rows (dense_smem() sizes it)
+    // dense-precision Gaussian only: P [dp][dp], then one row of pairs (x_j, x_j) per
+    // chain slot, after the reduction's rows (dense_smem() sizes it)
     float* dsm = nullptr;
     if constexpr (KIND == TGT_GAUSS_DENSE) {
         dsm = reinterpret_cast<float*>(
             (reinterpret_cast<uintptr_t>(s_q + (size_t)NQ * P.smax + NCS) + 15) & ~(uintptr_t)15);
-        for (int o = tid; o < (dp * dp + dp) / 4; o += blockDim.x)
+        for (int o = tid; o < dp * dp / 4; o += blockDim.x)
             reinterpret_cast<float4*>(dsm)[o] = reinterpret_cast<const float4*>(P.prec)[o];
     }
 
