@@ -46,6 +46,17 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     return r;
 }
 
+// 1 / x for x in [1, 2]: the hardware's approximation (within one ulp) and two Newton-
+// Raphson steps, each r + r (1 - x r).  Equal to the division 1.0f / x for every binary32
+// x of [1, 2] (tests/test_gpu_reciprocal.py goes through all of them), without its range
+// checks.
+__device__ __forceinline__ float rcp_1_2(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    r = fmaf(r, fmaf(-x, r, 1.0f), r);
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+
 // ---------------------------------------------------------------- Philox4x32-10
 // Ten rounds; each multiplies words 0 and 2 by the round multipliers, xors the
 // high halves into the other words with the round key, bumps the key by the

@@ -175,7 +175,8 @@ logreg_grad_f32_kernel(const float* __restrict__ W, int64_t M, const float* __re
 
 // ---------------------------------------------------------------- packed form
 // The same contraction for kp <= 128 with packed binary32 pairs (fma.rn.f32x2),
-// every sum in the plain kernel's order (the results are its results, but with ROUND).  What bounds
+// every sum in the plain kernel's order and every operation rounded as there, so that
+// without ROUND the results are the plain kernel's bit for bit.  What bounds
 // it is the FMA pipe: 2 M n d multiply-adds, of which the pipe retires 128 per clock
 // and SM either way, but a packed instruction carries two, so half the issue slots
 // are left for the operand loads and the epilogue.  A thread owns 8 chains x 4 rows
@@ -213,7 +214,7 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     float* Xs = Ws + (ROUND ? TM * LD : TM / 2 * LDW);  // [TN][LD]
     float* Rt = Xs + TN * LD;         // [TN][RTP]  Rt[row][32 i + 4 cr]: chain cr + 16 i twice, cr + 16 i + 8 twice
     float* wsq = Rt + TN * RTP;       // [TM] |w|^2
-    ff* s_lp = reinterpret_cast<ff*>(wsq + TM);  // [TM] log p of the upper half of the rows
+    ff* s_lp = reinterpret_cast<ff*>(wsq + TM);  // [8][2][32] log p of the upper half of the rows, a lane's chains
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t m0 = (int64_t)blockIdx.x * TM;
@@ -346,14 +347,7 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
                     for (int h = 0; h < 2; ++h) {
                         const float zz = h == 0 ? zp.x : zp.y;
                         const float t = expf(-fabsf(zz));               // e^{-|z|} in (0, 1]
-                        // 1 / (1 + t): the hardware reciprocal and two Newton steps round as the
-                        // division does for every 1 + t in [1, 2] but 2 - 2^-23 (checked
-                        // exhaustively from starts within two ulps)
-                        const float opt = 1.0f + t;
-                        float inv;
-                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(opt));
-                        inv = fmaf(inv, fmaf(-opt, inv, 1.0f), inv);
-                        inv = fmaf(inv, fmaf(-opt, inv, 1.0f), inv);
+                        const float inv = rcp_1_2(1.0f + t);
                         const float sig = zz >= 0.0f ? inv : t * inv;   // sigmoid(z)
                         r[h] = ok ? yn[e] - sig : 0.0f;
                         if constexpr (ROUND) {  // y z - max(z, 0); log(1 + t) below
@@ -397,13 +391,16 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
     }
 
     // ---- outputs: gradient partial (plus the prior on range 0) and log p partial.
-    // log p: the 8 lanes of a chain, then the two warps that share it, in a fixed order
+    // log p: row dc + 8's partial (the warp two up, same lane) before the 8 lanes of a
+    // chain, the order of the plain kernel's butterfly
+    ff* s_w = s_lp + 32 * (warp & 1) + lane;
+    if (warp >= 2)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) lacc[c] = group_sum_ff<8>(lacc[c]);
-    if (warp >= 2 && (lane & 7) == 0)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s_lp[cr + 8 * c] = lacc[c];
+        for (int c = 0; c < 8; ++c) s_w[64 * c] = lacc[c];
     __syncthreads();  // s_lp and wsq are visible (the loop may be empty)
+    if (warp < 2)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) lacc[c] = group_sum_ff<8>(ff_add(lacc[c], s_w[64 * c]));
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         const int64_t m = m0 + cr + 8 * c;
@@ -423,7 +420,7 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
             *reinterpret_cast<float4*>(gpart + ((size_t)s * M + m) * KP + col) = v;
         }
         if (warp < 2 && (lane & 7) == 0) {
-            ff l = ff_add(lacc[c], s_lp[cr + 8 * c]);
+            ff l = lacc[c];
             if (s == 0) l = ff_add(l, -0.5f * inv_v * wsq[cr + 8 * c]);
             lpart[(size_t)s * M + m] = make_float2(l.hi, l.lo);
         }
@@ -434,14 +431,15 @@ logreg_grad_f32p_kernel(const float* __restrict__ W, int64_t M, const float* __r
 // kp = 192 and above).  It takes the launch when some SM gets two blocks; below that an
 // SM holds one block, whose four warps reach 83 of the FMA pipe's 128 lanes a clock, and the
 // plain kernel's eight are faster (n = 262, d = 72, M = 198, 20 blocks: 15 steps of a run
-// 787 against 847 us).  Both give the same bits.
+// 787 against 847 us).  In the sampler both give the same bits, so the line between
+// them is of speed alone; a target call (ROUND) adds in another order in the packed one.
 template <int KP>
 constexpr bool kPacked = KP <= 128;
 
 template <int KP>
 size_t f32_smem(bool packed) {
     const size_t tiles = (size_t)TM * (KP + 4) + (size_t)TN * (KP + 4) + TM;
-    if (packed) return (tiles + (size_t)TN * RTP + 2 * TM) * sizeof(float);  // W: TM / 2 rows of 2 kp + 4
+    if (packed) return (tiles + (size_t)TN * RTP + 16 * TM) * sizeof(float);  // W: TM / 2 rows of 2 kp + 4
     return (tiles + (size_t)TN * RTS) * sizeof(float);
 }
 
