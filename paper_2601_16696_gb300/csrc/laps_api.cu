@@ -60,8 +60,8 @@ static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 // ------------------------------------------------------------------ small kernels
 __global__ void unpack_rows_kernel(const float* __restrict__ src, const float* __restrict__ scale,
-                                   float* __restrict__ dst, int64_t M, int d, int d_pad) {
-    unpack_rows(src, scale, dst, M, d, d_pad);
+                                   float* __restrict__ dst, RowIndex r, int d_pad) {
+    unpack_rows(src, scale, dst, r, d_pad);
 }
 __global__ void ff_to_double_kernel(const float2* __restrict__ src, double* __restrict__ dst,
                                     int64_t n) {
@@ -96,7 +96,8 @@ void launch_set_coefs(Coefs* dst, const Coefs& cf, cudaStream_t st) {
 }
 void launch_unpack(const float* src, const float* scale, float* dst, int64_t M, int d, int d_pad,
                    cudaStream_t st) {
-    unpack_rows_kernel<<<row_blocks(M), 256, 0, st>>>(src, scale, dst, M, d, d_pad);
+    const RowIndex r = row_index(M, d);
+    unpack_rows_kernel<<<row_blocks(r), 256, 0, st>>>(src, scale, dst, r, d_pad);
 }
 
 void coefs_table(Coefs& cf) {
@@ -692,8 +693,7 @@ laps_status laps_adapt_freeze(laps_ctx* c, int frozen) {
 laps_status laps_sample(const laps_ctx* c, float* x_out, void* stream) {
     if (!c || !x_out || !aligned(x_out, 4)) return fail(LAPS_ERR_INVALID_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    unpack_rows_kernel<<<row_blocks(c->M), 256, 0, st>>>(c->y, c->sigma, x_out, c->M, c->d,
-                                                             c->d_pad);
+    launch_unpack(c->y, c->sigma, x_out, c->M, c->d, c->d_pad, st);
     CK(cudaGetLastError());
     return LAPS_OK;
 }
@@ -707,8 +707,7 @@ laps_status laps_get_state(const laps_ctx* c, float* y, float* u, float* g, doub
     for (int k = 0; k < 3; ++k) {
         if (!dst[k]) continue;
         if (!aligned(dst[k], 4)) return fail(LAPS_ERR_INVALID_ARG, "misaligned output");
-        unpack_rows_kernel<<<row_blocks(c->M), 256, 0, st>>>(src[k], nullptr, dst[k], c->M,
-                                                                 c->d, c->d_pad);
+        launch_unpack(src[k], nullptr, dst[k], c->M, c->d, c->d_pad, st);
         CK(cudaGetLastError());
     }
     if (logp) {

@@ -203,9 +203,8 @@ __global__ void batch_start_kernel(KParams* probs, Hyper* hyper, int n, uint32_t
 // problem k's positions x = sigma o y, except after a switch that no proposal
 // followed (y is still in x then); the phase machine is read on the device
 __global__ void batch_unpack_kernel(const float* __restrict__ y, const float* __restrict__ sigma,
-                                    const Hyper* __restrict__ h, float* __restrict__ x, int64_t M, int d,
-                                    int d_pad) {
-    unpack_rows(y, h->phase == 1 && h->p == 0 ? nullptr : sigma, x, M, d, d_pad);
+                                    const Hyper* __restrict__ h, float* __restrict__ x, RowIndex r, int d_pad) {
+    unpack_rows(y, h->phase == 1 && h->p == 0 ? nullptr : sigma, x, r, d_pad);
 }
 
 laps_status read_hypers(laps_batch* b) {
@@ -546,8 +545,8 @@ laps_status laps_batch_sample(laps_batch* b, int k, float* x_out, void* stream) 
     if (!b || !x_out || k < 0 || k >= b->n || reinterpret_cast<uintptr_t>(x_out) % 4)
         return fail(LAPS_ERR_INVALID_ARG, "bad argument");
     const BProb& p = b->P[k];
-    batch_unpack_kernel<<<row_blocks(p.M), 256, 0, (cudaStream_t)stream>>>(p.y, p.sigma, b->hyper + k, x_out, p.M,
-                                                                  (int)p.d, p.d_pad);
+    const RowIndex r = row_index(p.M, (int)p.d);
+    batch_unpack_kernel<<<row_blocks(r), 256, 0, (cudaStream_t)stream>>>(p.y, p.sigma, b->hyper + k, x_out, r, p.d_pad);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LAPS_OK : cuda_fail(e, "laps_batch_sample");
 }

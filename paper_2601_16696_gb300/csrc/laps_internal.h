@@ -7,6 +7,7 @@
 
 #include "laps_logreg.cuh"
 #include "laps_params.h"
+#include "laps_rows.cuh"
 #include "laps_resident_kernel.cuh"
 
 struct laps_target {
@@ -81,28 +82,6 @@ struct laps_ctx {
 };
 
 namespace laps {
-// Rows of d_pad floats to rows of d (times scale, if any), a warp per row: no index
-// division, consecutive lanes on consecutive coordinates, four loads in flight a lane.
-__device__ __forceinline__ void unpack_rows(const float* __restrict__ src, const float* __restrict__ scale,
-                                            float* __restrict__ dst, int64_t M, int d, int d_pad) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; m < M; m += nw) {
-        const float* a = src + m * d_pad;
-        float* o = dst + m * d;
-        for (int i0 = lane; i0 < d; i0 += 128) {
-            float v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (i0 + 32 * u < d) v[u] = a[i0 + 32 * u] * (scale ? scale[i0 + 32 * u] : 1.0f);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (i0 + 32 * u < d) o[i0 + 32 * u] = v[u];
-        }
-    }
-}
-// blocks of 256 threads for M rows, a warp per row
-inline int row_blocks(int64_t M) { return (int)(M < 8 * 8192 ? (M + 7) / 8 : 8192); }
 laps_status fail(laps_status st, const std::string& msg);
 laps_status cuda_fail(cudaError_t e, const char* what);
 // Let kernel fn use at least `bytes` of dynamic shared memory.  The limit is a

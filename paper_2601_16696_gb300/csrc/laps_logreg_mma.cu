@@ -43,6 +43,7 @@
 
 #include "laps_device.cuh"
 #include "laps_logreg.cuh"
+#include "laps_rows.cuh"
 #include "laps_tc.cuh"
 
 namespace laps {
@@ -456,18 +457,16 @@ __global__ void pair_labels_kernel(const float* __restrict__ y, int n, int n32, 
 }
 
 // caller's points [M][d] -> the FP32 [M][kp] copy and the BF16 hi | lo [M_pad][2 kp] copy
-__global__ void pack_points_kernel(const float* __restrict__ x, int64_t M, int d, int kp,
-                                   float* __restrict__ W32, __nv_bfloat16* __restrict__ Wb) {
-    const int lane = threadIdx.x & 31;  // a warp per row: no index division
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; m < M; m += nw)
-        for (int i = lane; i < kp; i += 32) {
-            const float v = i < d ? x[m * d + i] : 0.0f;
-            W32[m * kp + i] = v;
+__global__ void pack_points_kernel(const float* __restrict__ x, RowIndex r, int d, float* __restrict__ W32,
+                                   __nv_bfloat16* __restrict__ Wb) {
+    for_elements(
+        r, [&](int64_t m, int i) { return i < d ? x[m * d + i] : 0.0f; },
+        [&](float v, int64_t k, int64_t m, int i) {
+            W32[k] = v;
             const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-            Wb[m * 2 * kp + i] = hi;
-            Wb[m * 2 * kp + kp + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
-        }
+            Wb[m * 2 * r.w + i] = hi;
+            Wb[m * 2 * r.w + r.w + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
+        });
 }
 
 template <int KP, bool FOLD>
@@ -483,9 +482,8 @@ cudaError_t launch_mma(const CUtensorMap& mw, const CUtensorMap& mx, const MmaAr
 
 cudaError_t logreg_pack_points(const float* x, int64_t M, int d, int kp, float* W32, void* Wb,
                                cudaStream_t st) {
-    const int blocks = (int)std::min<int64_t>((M + 7) / 8, 8192);  // 8 warps, so 8 rows, a block
-    pack_points_kernel<<<blocks, 256, 0, st>>>(x, M, d, kp, W32,
-                                                          reinterpret_cast<__nv_bfloat16*>(Wb));
+    const RowIndex r = row_index(M, kp);
+    pack_points_kernel<<<row_blocks(r), 256, 0, st>>>(x, r, d, W32, reinterpret_cast<__nv_bfloat16*>(Wb));
     return cudaGetLastError();
 }
 

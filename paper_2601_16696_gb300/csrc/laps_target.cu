@@ -64,37 +64,116 @@ __global__ void target_logp_grad_kernel(int kind, const float* __restrict__ x, i
     if (lane == 0) logp[m] = part.hi + part.lo;
 }
 
-// LOGREG: the caller's [M][d] points padded to the contraction layout and back, a warp
-// per row (no 64-bit index division: M = 8192, d = 101, tensor-core gradient calls
-// 121.2 -> 117.1 us and 216.5 -> 210.7 us)
-__global__ void logreg_pack_kernel(const float* __restrict__ x, float* __restrict__ W, int64_t M,
-                                   int d, int kp) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; m < M; m += nw)
-        for (int i = lane; i < kp; i += 32) W[m * kp + i] = i < d ? x[m * d + i] : 0.0f;
+// LOGREG: the caller's [M][d] points padded to the contraction layout and back (laps_rows.cuh)
+__global__ void logreg_pack_kernel(const float* __restrict__ x, float* __restrict__ W, RowIndex r, int d) {
+    for_elements(
+        r, [&](int64_t m, int i) { return i < d ? x[m * d + i] : 0.0f; },
+        [&](float v, int64_t k, int64_t, int) { W[k] = v; });
 }
-// the S partials of the gradient kernel summed in order, back to the caller's [M][d]
+// The S partials of the gradient kernel summed in order, back to the caller's [M][d].  The
+// first lp_blocks blocks add log p, a thread a point; the others add the gradient, with
+// sixteen loads in flight a thread, since a call of few points has up to 157 partials.
+// Measured, us a launch (a thread an element and four loads in flight; a warp a row, its
+// columns one after another; this), three-term form, n = 10^4, d = 101: M = 64 23, 68, 14.9;
+// M = 1000 10.8, 25.9, 8.9; M = 8192 11.3, 9.2, 8.8; FP32, M = 64 4.2, 8.4, 3.1.
+__device__ __forceinline__ void sum_logp(const float2* __restrict__ lp, float* __restrict__ logp, int64_t M, int S) {
+    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (m >= M) return;
+    ff l = ff_make(0.0f);
+    for (int s0 = 0; s0 < S; s0 += 8) {
+        float2 v[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            if (s0 + b < S) v[b] = lp[(size_t)(s0 + b) * M + m];
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            if (s0 + b < S) l = ff_add(l, ff{v[b].x, v[b].y});
+    }
+    logp[m] = l.hi + l.lo;
+}
+// rows of 32 columns and more: a warp takes 32 U columns of a row
+template <int U>
 __global__ void logreg_unpack_kernel(const float* __restrict__ G, const float2* __restrict__ lp,
                                      float* __restrict__ grad, float* __restrict__ logp, int64_t M,
-                                     int d, int kp, int S) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const size_t stride = (size_t)M * kp;
-    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; m < M; m += nw) {
-        for (int i = lane; i < d; i += 32) {
-            const float* src = G + m * kp + i;
-            float g = 0.0f;
-#pragma unroll 4
-            for (int s = 0; s < S; ++s) g += src[s * stride];
-            grad[m * d + i] = g;
-        }
-        if (lane == 0) {
-            ff l = ff_make(0.0f);
-            for (int s = 0; s < S; ++s) l = ff_add(l, ff{lp[(size_t)s * M + m].x, lp[(size_t)s * M + m].y});
-            logp[m] = l.hi + l.lo;
-        }
+                                     int d, int kp, int S, int lp_blocks) {
+    constexpr int B = 16 / U;
+    if ((int)blockIdx.x < lp_blocks) {
+        if (blockIdx.y == 0) sum_logp(lp, logp, M, S);
+        return;
     }
+    const int i0 = 32 * U * blockIdx.y + (threadIdx.x & 31);
+    const int64_t w0 = ((int64_t)blockIdx.x - lp_blocks) * 8 + (threadIdx.x >> 5), nw = ((int64_t)gridDim.x - lp_blocks) * 8;
+    const size_t stride = (size_t)M * kp;
+    for (int64_t m = w0; m < M; m += nw) {
+        const float* src = G + m * kp + i0;
+        float g[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) g[u] = 0.0f;
+        for (int s0 = 0; s0 < S; s0 += B) {
+            float v[B][U];
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (s0 + b < S && i0 + 32 * u < d) v[b][u] = src[(s0 + b) * stride + 32 * u];
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (s0 + b < S && i0 + 32 * u < d) g[u] += v[b][u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + 32 * u < d) grad[m * d + i0 + 32 * u] = g[u];
+    }
+}
+// shorter rows: a thread an element of the flat array
+template <int B>
+__global__ void logreg_unpack_short_kernel(const float* __restrict__ G, const float2* __restrict__ lp,
+                                           float* __restrict__ grad, float* __restrict__ logp, RowIndex r, int64_t M,
+                                           int kp, int S, int lp_blocks) {
+    if ((int)blockIdx.x < lp_blocks) {
+        sum_logp(lp, logp, M, S);
+        return;
+    }
+    const size_t stride = (size_t)M * kp;
+    const int64_t step = ((int64_t)gridDim.x - lp_blocks) * blockDim.x;
+    for (int64_t k = ((int64_t)blockIdx.x - lp_blocks) * blockDim.x + threadIdx.x; k < r.n; k += step) {
+        const int64_t m = r.n <= 0x7fffffff ? (int64_t)(((uint64_t)k * r.m) >> r.s) : k / r.w;
+        const float* src = G + m * kp + (k - m * r.w);
+        float g = 0.0f;
+        for (int s0 = 0; s0 < S; s0 += B) {
+            float v[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+                if (s0 + b < S) v[b] = src[(s0 + b) * stride];
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+                if (s0 + b < S) g += v[b];
+        }
+        grad[k] = g;
+    }
+}
+void launch_pack(const float* x, float* W, int64_t M, int d, int kp, cudaStream_t st) {
+    const RowIndex r = row_index(M, kp);
+    logreg_pack_kernel<<<row_blocks(r), 256, 0, st>>>(x, W, r, d);
+}
+void launch_unpack_grad(const float* G, const float2* lp, float* grad, float* logp, int64_t M, int d, int kp, int S,
+                        cudaStream_t st) {
+    const int lp_blocks = (int)((M + 255) / 256);
+    if (d < 32) {
+        const RowIndex r = row_index(M, d);
+        auto fn = S > 4 ? logreg_unpack_short_kernel<16> : logreg_unpack_short_kernel<2>;
+        fn<<<lp_blocks + (int)std::min<int64_t>((r.n + 255) / 256, 4096), 256, 0, st>>>(G, lp, grad, logp, r, M, kp, S, lp_blocks);
+        return;
+    }
+    // four columns a lane (and fewer partials at once) where the rows alone fill the GPU, or
+    // where few partials would leave most of the sixteen loads unused: M = 2500, d = 128 and 22
+    // partials 6.9 us with one column against 9.1 with four; M = 1500, d = 300 and one 7.5, 3.2
+    const int U = M >= 4096 || (M >= 1024 && S <= 4) ? 4 : 1;
+    const dim3 grid(lp_blocks + (unsigned)std::min<int64_t>((M + 7) / 8, 8192), (unsigned)((d + 32 * U - 1) / (32 * U)));
+    auto fn = U == 4 ? logreg_unpack_kernel<4> : logreg_unpack_kernel<1>;
+    fn<<<grid, 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S, lp_blocks);
 }
 
 // USER targets: the callback's FP32 log p as the float-float partial the chain
@@ -131,11 +210,10 @@ static laps_status streamed_logp_grad(const laps_target* tg, const float* x, int
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&lp, (size_t)S * M * 8, st);
     laps_status rs = LAPS_OK;
     if (e == cudaSuccess) {
-        const int blocks = row_blocks(M);
-        logreg_pack_kernel<<<blocks, 256, 0, st>>>(x, W, M, d, kp);
+        launch_pack(x, W, M, d, kp, st);
         rs = streamed_target_grad(tg, W, M, S, G, lp, st);
         if (rs == LAPS_OK) {
-            logreg_unpack_kernel<<<blocks, 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S);
+            launch_unpack_grad(G, lp, grad, logp, M, d, kp, S, st);
             e = cudaGetLastError();
         }
     }
@@ -175,7 +253,7 @@ static laps_status logreg_logp_grad_mixed(const laps_target* tg, const float* x,
     if (e == cudaSuccess) e = logreg_mma_wmap(tmW, Wb, M_pad, kp);
     if (e == cudaSuccess) e = logreg_grad_mma(L, tmW, W32, M, S, rps, L.bin, G, lp, tg->status, 2000000000LL, st);
     if (e == cudaSuccess) {
-        logreg_unpack_kernel<<<row_blocks(M), 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S);
+        launch_unpack_grad(G, lp, grad, logp, M, d, kp, S, st);
         e = cudaGetLastError();
     }
     if (W32) cudaFreeAsync(W32, st);
@@ -204,14 +282,13 @@ static laps_status logreg_logp_grad_x3(const laps_target* tg, const float* x, in
     cudaError_t e = cudaMallocAsync((void**)&W32, (size_t)M * kp * 4, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&G, (size_t)S * M * kp * 4, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&lp, (size_t)S * M * 8, st);
-    const int blocks = row_blocks(M);
     if (e == cudaSuccess) {
-        logreg_pack_kernel<<<blocks, 256, 0, st>>>(x, W32, M, d, kp);
+        launch_pack(x, W32, M, d, kp, st);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = logreg_grad_x3(L, W32, M, S, rps, G, lp, tg->status, 2000000000LL, st);
     if (e == cudaSuccess) {
-        logreg_unpack_kernel<<<blocks, 256, 0, st>>>(G, lp, grad, logp, M, d, kp, S);
+        launch_unpack_grad(G, lp, grad, logp, M, d, kp, S, st);
         e = cudaGetLastError();
     }
     if (W32) cudaFreeAsync(W32, st);
