@@ -212,12 +212,11 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
         if (warp == 1) {
             constexpr uint32_t ID_Z = idesc_bf16(MT, TNR);
             const uint64_t dX = sw128_desc(sX), dW = sw128_desc(sW);
-            ok = __all_sync(0xffffffffu, mbar_wait(bar(B_WFULL), 0, deadline));
+            ok = mbar_wait_warp(bar(B_WFULL), 0, deadline);
             for (int c = 0; c < nc && ok; ++c) {
                 const int st = c % NSTAGE, zb = c & 1;
-                ok = mbar_wait(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) &&
-                     mbar_wait(bar(B_ZEMPTY + zb), ((c >> 1) & 1) ^ 1, deadline);
-                ok = __all_sync(0xffffffffu, ok);
+                ok = mbar_wait_warp(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) &&
+                     mbar_wait_warp(bar(B_ZEMPTY + zb), ((c >> 1) & 1) ^ 1, deadline);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t bX = dX + (uint64_t)((uint32_t)st * S::STAGE >> 4);
@@ -240,9 +239,8 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
             const uint64_t dXmn = sw128_mn_desc(sX, S::ATOM);
             for (int c = 0; c < nc && ok; ++c) {
                 const int rb = c & 1, st = c % NSTAGE;
-                ok = mbar_wait(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) &&
-                     mbar_wait(bar(B_RFULL + rb), (c >> 1) & 1, deadline);
-                ok = __all_sync(0xffffffffu, ok);
+                ok = mbar_wait_warp(bar(B_XFULL + st), (c / NSTAGE) & 1, deadline) &&
+                     mbar_wait_warp(bar(B_RFULL + rb), (c >> 1) & 1, deadline);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t aR = tR + (uint32_t)rb * (TNR / 2);
@@ -281,7 +279,7 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
         bool ok = true;
         for (int c = grp; c < nc && ok; c += 2) {
             const int zb = grp, rb = grp;  // Z and R buffers of this group
-            if (!mbar_wait(bar(B_ZFULL + zb), (c >> 1) & 1, deadline)) { ok = false; break; }
+            if (!mbar_wait_warp(bar(B_ZFULL + zb), (c >> 1) & 1, deadline)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int pass = 0; pass < 2; ++pass) {
@@ -361,7 +359,7 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
                 const float2 ls = unpack2(lsum);
                 lp = ff_add(ff_add(lp, ls.x), ls.y);
             }
-            if (pass == 0 && !mbar_wait(bar(B_REMPTY + rb), ((c >> 1) & 1) ^ 1, deadline)) { ok = false; break; }
+            if (pass == 0 && !mbar_wait_warp(bar(B_REMPTY + rb), ((c >> 1) & 1) ^ 1, deadline)) { ok = false; break; }
             // R row rt, data rows col0 .. col0 + 31 of the chunk: columns col0 / 2 .. of this lane's R buffer
             tmem_st16(tR + lane_off + (uint32_t)(rb * (TNR / 2) + col0 / 2), pr);
             }
@@ -371,8 +369,7 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_RFULL + rb));
         }
-        if (ok && !mbar_wait(bar(B_GDONE), 0, deadline)) ok = false;
-        ok = __all_sync(0xffffffffu, ok);
+        ok = ok && mbar_wait_warp(bar(B_GDONE), 0, deadline);
         const int64_t m = m0 + rt;
         const float* wrow = A.W32 + (size_t)(m < A.M ? m : 0) * KP;
         if (!ok) atomicExch(&s_fail, 1);

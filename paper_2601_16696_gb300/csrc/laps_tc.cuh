@@ -44,6 +44,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
         if ((k & 63u) == 63u && global_ns() > deadline) return false;
     }
 }
+// The same for a whole warp, one outcome for all its lanes.  Each lane polls for itself, so at
+// the deadline some may have seen the phase and others not; one that gave up alone would leave
+// the rest to run .sync.aligned instructions and full-mask warp barriers without it, which is
+// undefined and may never end.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, unsigned long long deadline) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, deadline));
+}
 // Bound of the waits after a failure, for the copies and MMAs a CTA issued
 // itself: at least a second whatever the caller's timeout, so that a CTA never
 // frees its tensor memory or exits while its own asynchronous work is in flight
