@@ -192,14 +192,14 @@ logreg_grad_mma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_con
                 tma_load_2d(dst + (uint32_t)a * S::ATOM, &tmX, 64 * a, row, bar(B_XFULL + st));  // rows past n: 0
             issued = c + 1;
         }
-        if (!ok) {
-            atomicExch(&s_fail, 1);
-            // wait (bounded) for the copies this thread issued
-            const unsigned long long d2 = global_ns() + drain_ns(A.timeout_ns);
-            mbar_wait(bar(B_WFULL), 0, d2);
-            for (int c = max(0, issued - NSTAGE); c < issued; ++c)
-                mbar_wait(bar(B_XFULL + c % NSTAGE), (c / NSTAGE) & 1, d2);
-        }
+        if (!ok) atomicExch(&s_fail, 1);
+        // wait (bounded) for the copies this thread issued, whatever the other roles did: one of
+        // them may have given up before it waited for the last chunks, and a CTA must not end
+        // while copies into its shared memory are in flight
+        const unsigned long long d2 = global_ns() + drain_ns(A.timeout_ns);
+        mbar_wait(bar(B_WFULL), 0, d2);
+        for (int c = max(0, issued - NSTAGE); c < issued; ++c)
+            mbar_wait(bar(B_XFULL + c % NSTAGE), (c / NSTAGE) & 1, d2);
       }
       __syncwarp();
     } else if (warp <= 2) {

@@ -25,6 +25,18 @@ def test_warp_wide_roles_wait_as_one(name):
     assert len(re.findall(r"\bmbar_wait_warp\(", roles)) == 8
 
 
+@pytest.mark.parametrize("name", ["laps_logreg_mma.cu", "laps_logreg_x3.cu"])
+def test_the_copying_warp_always_waits_for_its_copies(name):
+    """Also when it issued every chunk itself and another role gave up: the waits for the last chunks stand in no
+    condition (the producer's block has no branch after its loop but the one that records the failure)."""
+    with open(os.path.join(CSRC, name)) as f:
+        src = re.sub(r"//[^\n]*", "", f.read())
+    role = src[src.index("tma_load_2d(dst"):src.index("} else if (warp <= 2) {")]
+    after = role[role.index("issued = c + 1;"):]
+    assert after.count("if (") == 1 and "if (!ok) atomicExch(&s_fail, 1);" in after
+    assert re.search(r"for \(int c = max\(0, issued - \w+\); c < issued; \+\+c\)\s*mbar_wait\(", after)
+
+
 def test_the_warp_wide_wait_votes():
     with open(os.path.join(CSRC, "laps_tc.cuh")) as f:
         src = f.read()
