@@ -56,6 +56,7 @@ struct laps_ctx {
     float* ulp = nullptr;            // USER targets: the callback's FP32 log p [M]
     float2 *dlw = nullptr, *lpw = nullptr, *lpart = nullptr;
     int* go = nullptr;
+    bool seg_ahead = false;          // chain updates load their inputs a chain ahead (laps_streamed.cu)
     int nsplit = 1, seg_cpl = 0, seg_G = 0, fin_G = 0, adj_integ = 0;
     size_t seg_smem = 0, fin_slice_smem = 0, fin_gather_smem = 0;
     laps::Hyper* h_hyper = nullptr;  // pinned host copy of the phase machine (owned)

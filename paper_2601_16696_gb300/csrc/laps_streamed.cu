@@ -34,8 +34,9 @@ constexpr int kSegWarps = kSegThreads / 32;
 constexpr int kFinThreads = 256;
 
 // ---------------------------------------------------------------- chain update
-template <int CPL>
-__global__ void __launch_bounds__(kSegThreads, CPL <= 4 ? 2 : 1) seg_kernel(const KParams P, const SegOp op) {
+// AHEAD: a chain's inputs are loaded while the previous chain is updated (fetch below)
+template <int CPL, bool AHEAD>
+__global__ void __launch_bounds__(kSegThreads, CPL > 4 ? 1 : AHEAD ? 2 : 3) seg_kernel(const KParams P, const SegOp op) {
     constexpr int NB = CPL / 4;
     extern __shared__ __align__(16) float seg_smem[];
     __shared__ Hyper H;
@@ -146,9 +147,8 @@ __global__ void __launch_bounds__(kSegThreads, CPL <= 4 ? 2 : 1) seg_kernel(cons
     // come with them; more are read where they are used.  M = 8192, d = 101: the update that
     // closes a mixed step 15.5 -> 13.8 us.  (More coordinates a lane: no gain measured at
     // d = 300, and the registers are short.)
-    constexpr bool kAhead = CPL <= 4;
     const bool run = op.init == 0;
-    const bool g_ahead = kAhead && (op.first || (op.after_grad && P.nsplit <= 2));
+    const bool g_ahead = AHEAD && (op.first || (op.after_grad && P.nsplit <= 2));
     struct Ahead {
         float y[CPL], u[CPL], g0[CPL], g1[CPL];
         float2 l, e, l0, l1;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kSegThreads, CPL <= 4 ? 2 : 1) seg_kernel(cons
         }
     };
     Ahead A;
-    if (kAhead && run && mb0 + warp < mb1) fetch(mb0 + warp, A);
+    if (AHEAD && run && mb0 + warp < mb1) fetch(mb0 + warp, A);
 
     for (int m = mb0 + warp; m < mb1; m += kSegWarps) {
         const uint32_t mg = (uint32_t)(m + P.m0);  // the chain's index in the whole ensemble
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kSegThreads, CPL <= 4 ? 2 : 1) seg_kernel(cons
             store(P.g, m, g);
             if (lane == 0) P.logp_ff[m] = make_float2(lp.hi, lp.lo);
         } else {
-            if (!kAhead) fetch(m, A);
+            if (!AHEAD) fetch(m, A);
             ff lpn = ff_make(0.0f);
 #pragma unroll
             for (int q = 0; q < CPL; ++q) {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kSegThreads, CPL <= 4 ? 2 : 1) seg_kernel(cons
                     for (int q = 0; q < CPL; ++q) g[q] = sg[q] * (P.nsplit == 2 ? A.g0[q] + A.g1[q] : A.g0[q]);
                 }
             }
-            if (kAhead && m + kSegWarps < mb1) fetch(m + kSegWarps, A);
+            if (AHEAD && m + kSegWarps < mb1) fetch(m + kSegWarps, A);
             if (!g_ahead) {
                 if (op.first) load(P.g, m, g);
                 else if (op.after_grad) load_grad(m, g, lpn);
@@ -452,18 +452,18 @@ __global__ void precondition_kernel(const KParams P) {
 // ---------------------------------------------------------------- host
 namespace {
 
-const void* seg_fn(int cpl) {
-    switch (cpl) {
-    case 4: return (const void*)seg_kernel<4>;
-    case 8: return (const void*)seg_kernel<8>;
-    case 16: return (const void*)seg_kernel<16>;
+const void* seg_fn(const laps_ctx* c) {
+    switch (c->seg_cpl) {
+    case 4: return c->seg_ahead ? (const void*)seg_kernel<4, true> : (const void*)seg_kernel<4, false>;
+    case 8: return (const void*)seg_kernel<8, false>;
+    case 16: return (const void*)seg_kernel<16, false>;
     }
     return nullptr;
 }
 
 laps_status launch_seg(laps_ctx* c, const KParams& P, const SegOp& op, cudaStream_t st) {
     void* args[] = {const_cast<KParams*>(&P), const_cast<SegOp*>(&op)};
-    cudaError_t e = cudaLaunchKernel(seg_fn(c->seg_cpl), dim3(c->seg_G), dim3(kSegThreads), args,
+    cudaError_t e = cudaLaunchKernel(seg_fn(c), dim3(c->seg_G), dim3(kSegThreads), args,
                                      c->seg_smem, st);
     return e == cudaSuccess ? LAPS_OK : cuda_fail(e, "seg_kernel");
 }
@@ -630,8 +630,13 @@ laps_status streamed_setup(laps_ctx* c) {
     const int64_t g1 = (c->M + kSegWarps - 1) / kSegWarps, g4 = (c->M + 4 * kSegWarps - 1) / (4 * kSegWarps);
     c->seg_G = (int)std::min<int64_t>(g1, std::max<int64_t>(g4, nsm));
     c->G = c->seg_G;
+    // Loading a chain ahead takes 128 registers, so two blocks an SM; more blocks than that run
+    // three an SM with 80.  Updates of a mixed step, us, ahead and not: M = 10000 (313 blocks)
+    // 17.0 + 20.7 and 13.0 + 16.6, M = 32768 33.2 + 40.6 and 26.8 + 36.2; M = 8192 (256 blocks)
+    // 13.8 and 15.5 for the closing one.
+    c->seg_ahead = c->seg_cpl == 4 && c->seg_G <= 2 * nsm;
     c->seg_smem = (size_t)NQ * kSegWarps * dp * sizeof(float) + (size_t)kSegWarps * NCS * sizeof(ff);
-    e = ensure_dyn_smem((const void*)seg_fn(c->seg_cpl), c->seg_smem);
+    e = ensure_dyn_smem(seg_fn(c), c->seg_smem);
     if (e != cudaSuccess) return cuda_fail(e, "seg_kernel attribute");
     c->fin_G = std::max(1, std::min(2 * nsm, c->d));
     c->smax = (c->d + c->fin_G - 1) / c->fin_G;
