@@ -141,7 +141,8 @@ static size_t resident_smem(int d_pad, int threads, int lpc, int smax, int K, in
     return b + fullrank_smem(d_pad, slots, smax, K, threads);
 }
 
-laps_status choose_shape(laps_ctx* c) {
+// spread: smaller blocks where they fit one per SM (twice the blocks' columns in memory)
+laps_status choose_shape(laps_ctx* c, bool spread) {
     int dev;
     CK(cudaGetDevice(&dev));
     int nsm;
@@ -193,7 +194,7 @@ laps_status choose_shape(laps_ctx* c) {
     // against 10.7 / 46; M = 256 11.8 / 66 against 11.0 / 46; d = 10, M = 256 9.2 / 41 against
     // 8.6 / 29; d = 300, M = 1000 21.6 / 162 against 18.5 / 125.  128 threads gain a tenth of a
     // proposal and lose a tenth of an unadjusted iteration.
-    if (c->cfg.chains_per_block == 0 && c->cfg.dtilde_K == 0)
+    if (spread && c->cfg.chains_per_block == 0 && c->cfg.dtilde_K == 0)
         for (int k = 0; k < n_ok; ++k)
             if (ok[k].lpc == best.lpc && ok[k].cpl == best.cpl && ok[k].threads == 256 && best.threads > 256 &&
                 ok[k].G <= nsm)

@@ -90,7 +90,7 @@ laps_status cuda_fail(cudaError_t e, const char* what);
 // that needs less must not lower it under another live context's launches.
 cudaError_t ensure_dyn_smem(const void* fn, size_t bytes);
 // shared by the context API and the allocation-free entry point (laps_api.cu)
-laps_status choose_shape(laps_ctx* c);
+laps_status choose_shape(laps_ctx* c, bool spread = true);
 laps_status start_run(laps_ctx* c, const float* x0, float x0_scale, cudaStream_t st);
 laps_status launch_resident(laps_ctx* c, int mode, int n_iters, const float* x0, float x0_scale,
                             cudaStream_t st);

@@ -134,10 +134,16 @@ extern "C" laps_status laps_run_noalloc(const laps_target_desc* desc, int64_t M,
     c.d_pad = t.d_pad;
     c.T = std::max(2, (int)std::ceil(cfg->window_frac * (double)cfg->n_total_steps));
     c.trace_cap = 0;  // no trace: laps_stats reports the outcome
-    laps_status st = choose_shape(&c);
-    if (st != LAPS_OK) return st;
+    // the columns of a spread shape's blocks may be what no longer fits: then the fewest blocks
+    laps_status st = LAPS_OK;
     Carver count{nullptr, 0};
-    carve(c, t, count);
+    for (const bool spread : {true, false}) {
+        st = choose_shape(&c, spread);
+        if (st != LAPS_OK) return st;
+        count.off = 0;
+        carve(c, t, count);
+        if (count.off <= kNoAllocScratchBytes) break;
+    }
     if (count.off > kNoAllocScratchBytes)
         return fail(LAPS_ERR_INVALID_ARG,
                     "laps_run_noalloc: this problem needs " + std::to_string(count.off) +
